@@ -126,7 +126,11 @@ typedef struct {
 
 typedef struct tt_context tt_context;
 /* Factor of the merged core in the first sweep of every rounding (tt_round, tt_step).
- * TT_ROUND_TSQR: Householder TSQR (the SVD-based rounding of Sec. 3.1; the default).
+ * TT_ROUND_TSQR: the triangular factor of the SVD-based rounding of Sec. 3.1 (the default), to the
+ * accuracy of the arithmetic: from exact Gram products of the columns on the tensor cores (integer
+ * digits, a Cholesky factor in 128-bit fixed point), or by Householder TSQR where
+ * tt_context_set_tsqr chose its kernels, where the shape does not fit the former, or where its larger
+ * workspace cannot be had.
  * TT_ROUND_GRAM: Gram-based (Sec. 3.1 lists it among the solver's rounding methods): the FP64 Gram
  * matrix G = A^T A of the merged core's unfolding (virtual transport sum included) and a square
  * root R of G (R^T R = G, diagonally pivoted Cholesky) replace the TSQR's R; the rest of the
@@ -197,9 +201,10 @@ tt_status tt_context_set_rounding(tt_context *ctx, tt_rounding method);
 tt_status tt_context_set_sketch(tt_context *ctx, const double *omega_dev, int32_t nang, int32_t ell);
 
 /* Kernels of the tall-skinny QR over the merged core (the first sweep of the rounding, Sec. 3.1
- * footnote), per pass shape: for passes of ncap columns at precision prec (TT_PREC_FP64: FP64
- * passes; TT_PREC_MIXED: FP32 passes):
- *   variant 0: one thread per column (the default; at most 256 threads, i.e. ncap <= 256);
+ * footnote), per pass shape: passes of ncap columns at precision prec (TT_PREC_FP64: FP64 passes;
+ * TT_PREC_MIXED: FP32 passes) then run a Householder TSQR; without an entry for the shape they take
+ * the factor from exact Gram products (TT_ROUND_TSQR):
+ *   variant 0: one thread per column (at most 256 threads, i.e. ncap <= 256);
  *   variant 1: four lanes per column, each holding a quarter of the rows of a block (4 ncap <= 1024);
  *   variant 2: FP32 only, one thread per column over 32-row blocks with registers held so that
  *              four CTAs share an SM (ncap <= 160);
@@ -210,8 +215,9 @@ tt_status tt_context_set_sketch(tt_context *ctx, const double *omega_dev, int32_
  * merge tree over the leaves' R factors runs four lanes per column in every variant when
  * 4 ncap <= 1024.  leaves = cap on the TSQR leaves: <= 0 gives the default wave (2 CTAs per SM for
  * FP64, 3 for FP32); larger caps are clamped to 6 per SM.  The choice changes the order of
- * rounding errors only.  ncap <= 0 clears every entry.  tt_context_get_tsqr reports what a pass
- * of ncap columns would run.  The paper has no counterpart: these are launch-shape choices. */
+ * rounding errors only.  ncap <= 0 clears every entry.  tt_context_get_tsqr reports the Householder
+ * kernels of a pass of ncap columns: its entry, or the ones a pass without an entry falls back to.  The
+ * paper has no counterpart: these are launch-shape choices. */
 tt_status tt_context_set_tsqr(tt_context *ctx, tt_precision prec, int32_t ncap, int32_t variant, int32_t leaves);
 tt_status tt_context_get_tsqr(const tt_context *ctx, tt_precision prec, int32_t ncap, int32_t *variant,
                               int32_t *leaves);
@@ -238,7 +244,9 @@ tt_status tt_tsqr_geometry(tt_precision prec, int32_t variant, int32_t ncap, int
  * and the source pass (rcap_1 + 1 columns).  Each candidate (variant x leaf cap, one pass at a
  * time, the other at its best so far) is timed with CUDA events over `steps` (1..64) tt_steps,
  * after one untimed step, on a device copy of I; I itself is not modified, and a coupled plan's
- * material temperature is restored afterwards.  The fastest entries are stored in the context.
+ * material temperature is restored afterwards.  The fastest entries are stored in the context; where
+ * the default (no entry) is the fastest, the shape is left without an entry and reported as variant
+ * 0 with the default wave.
  * Synchronous; allocates the copy with cudaMalloc, so never under stream capture (TT_ERR_ARG).
  * chosen[4] (host, nullable): variant and leaf cap of the transport pass, then of the source
  * pass; ms[2] (host, nullable): ms per step with the defaults and with the choice.  Only the

@@ -70,14 +70,29 @@ tt_status ensure_ws(tt_context* ctx, size_t need) {
   return TT_OK;
 }
 
+// Size the workspace by a dry run of `fn(Bump&)` and provide it.  Where it cannot be had (a capture in
+// progress on a smaller workspace, or no memory), the call takes the Householder factors instead of
+// the exact Gram products, whose digit records need more (ctx->no_xg, cleared by the next call).
+template <class F>
+tt_status size_ws(tt_context* ctx, F&& fn) {
+  tt_status st = TT_OK;
+  for (int attempt = 0; attempt < 2; ++attempt) {
+    ctx->no_xg = attempt;
+    ttk::Bump dry{nullptr, 0, 0, true};
+    st = fn(dry);
+    if (st != TT_OK) return st;
+    st = ensure_ws(ctx, dry.need());
+    if (st == TT_OK) return st;
+    (void)cudaGetLastError();
+  }
+  return st;
+}
+
 // Run `fn(Bump&)` once as a dry run to size the workspace, then for real.
 template <class F>
 tt_status with_ws(tt_context* ctx, F&& fn) {
   InstrGuard guard(ctx);
-  ttk::Bump dry{nullptr, 0, 0, true};
-  tt_status st = fn(dry);
-  if (st != TT_OK) return st;
-  st = ensure_ws(ctx, dry.off);
+  const tt_status st = size_ws(ctx, fn);
   if (st != TT_OK) return st;
   ttk::Bump real{static_cast<char*>(ctx->ws), 0, ctx->ws_bytes, false};
   return fn(real);
@@ -105,7 +120,7 @@ struct StepGraph {
   double* energy = nullptr;
   void* ws = nullptr;
   size_t ws_bytes = 0;
-  int rounding = 0, sketch_nang = 0, sketch_ell = 0, coop_grid_max = 0, tsqr_leaf_cap = 0;
+  int rounding = 0, sketch_nang = 0, sketch_ell = 0, coop_grid_max = 0, tsqr_leaf_cap = 0, no_xg = 0;
   const double* sketch = nullptr;
   unsigned long tune_epoch = 0;
   // result of the capture
@@ -136,6 +151,7 @@ struct StepGraph {
     g.sketch_ell = ctx->sketch_ell;
     g.coop_grid_max = ctx->coop_grid_max;
     g.tsqr_leaf_cap = ctx->tsqr_leaf_cap;
+    g.no_xg = ctx->no_xg;
     g.tune_epoch = ttk::tune_of(ctx)->epoch;
     return g;
   }
@@ -143,7 +159,7 @@ struct StepGraph {
     if (plan != o.plan || plan_serial != o.plan_serial || d != o.d || dtype != o.dtype || rank != o.rank || tol != o.tol || rmax != o.rmax ||
         prec != o.prec || energy != o.energy || ws != o.ws || ws_bytes != o.ws_bytes || rounding != o.rounding ||
         sketch != o.sketch || sketch_nang != o.sketch_nang || sketch_ell != o.sketch_ell ||
-        coop_grid_max != o.coop_grid_max || tsqr_leaf_cap != o.tsqr_leaf_cap || tune_epoch != o.tune_epoch)
+        coop_grid_max != o.coop_grid_max || tsqr_leaf_cap != o.tsqr_leaf_cap || no_xg != o.no_xg || tune_epoch != o.tune_epoch)
       return false;
     for (int j = 0; j < TT_MAX_CORES; ++j)
       if (core[j] != o.core[j]) return false;
@@ -493,10 +509,7 @@ tt_status tt_step(tt_context* ctx, const tt_plan* plan, tt_tensor* I, double tol
   // the same key, or capture it now (the capture runs no kernel; launching the graph does).
   {
     InstrGuard guard(ctx);
-    ttk::Bump dry{nullptr, 0, 0, true};
-    st = body(dry);
-    if (st != TT_OK) return st;
-    st = ensure_ws(ctx, dry.off);
+    st = size_ws(ctx, body);
     if (st != TT_OK) return st;
   }
   const StepGraph key = StepGraph::of(ctx, plan, I, tol, rmax, prec, energy_dev);
@@ -601,6 +614,7 @@ tt_status tt_workspace_query(tt_context* ctx, const tt_plan* plan, const tt_tens
   tt_status st = check_tensor(x);
   if (st != TT_OK) return st;
   ttk::Bump dry{nullptr, 0, 0, true};
+  ctx->no_xg = 0;
   tt_tensor tmp = *x;
   if (plan) {
     st = check_plan_tensor(plan, x);
@@ -619,7 +633,7 @@ tt_status tt_workspace_query(tt_context* ctx, const tt_plan* plan, const tt_tens
       st = (x->dtype == TT_F64) ? ttk::round_impl<double, double>(ctx, &tmp, 1e-6, 1, dry)
                                 : ttk::round_impl<float, double>(ctx, &tmp, 1e-6, 1, dry);
   }
-  *bytes = dry.off;
+  *bytes = dry.need();
   return st;
 }
 

@@ -10,6 +10,7 @@
 #include "common.cuh"
 #include "instr.cuh"
 #include "step.cuh"
+#include "tune.cuh"
 
 struct tt_batch {
   tt_context* ctx;
@@ -32,6 +33,7 @@ struct tt_batch {
   cudaGraphExec_t exec;
   bool warmed;  // the first batched step ran eagerly (the graph is captured at the next one)
   cudaEvent_t pre, post;  // order the eager step after / before the context stream's work
+  ttk::TsqrTune tune;  // the context's kernel choice when the batch was made
   ttk::Instr counts;  // launch counts of the captured step (timing off)
 };
 
@@ -174,34 +176,45 @@ tt_status tt_batch_create(tt_context* ctx, int32_t nprob, const tt_plan* const* 
   size_t total = 0;
   double rows_all = 0.0;
   for (int i = 0; i < nprob; ++i) rows_all += (double)b->states[i].n[0];
+  // the kernel choice as it is now: the workspace below is sized for it
+  b->tune = *ttk::tune_of(ctx);
   ttk::Instr* prev = ttk::g_instr;
   ttk::g_instr = &b->counts;
-  for (int i = 0; i < nprob; ++i) {
-    tt_context& c = b->sub[i];
-    c.stream = b->streams[b->stream_of[i]];
-    c.ctrl = b->ctrls + i;
-    c.ws = nullptr;
-    c.ws_bytes = 0;
-    c.instr = &b->counts;
-    c.coop_grid_max = 1;
-    // TSQR leaves in proportion to the problem's share of the batch's rows (all problems run at
-    // once): at least 8, at most the single-problem wave
-    const double share = (double)b->states[i].n[0] / rows_all;
-    int cap = (int)(share * 3.0 * ctx->num_sms + 0.5);
-    c.tsqr_leaf_cap = cap < 8 ? 8 : cap;
-    ttk::Bump dry{nullptr, 0, 0, true};
-    tt_status st = step_dispatch(&c, b->plans[i], &b->states[i], b->tol[i], b->rmax[i], prec, dry);
-    if (st != TT_OK) {
-      ttk::g_instr = prev;
-      release(b);
-      return st;
+  for (int attempt = 0; attempt < 2 && !b->ws; ++attempt) {
+    total = 0;
+    for (int i = 0; i < nprob; ++i) {
+      tt_context& c = b->sub[i];
+      c.stream = b->streams[b->stream_of[i]];
+      c.ctrl = b->ctrls + i;
+      c.ws = nullptr;
+      c.ws_bytes = 0;
+      c.instr = &b->counts;
+      c.tune = &b->tune;
+      c.no_xg = attempt;  // where the exact Gram products' digit records do not fit: Householder factors
+      c.coop_grid_max = 1;
+      // TSQR leaves in proportion to the problem's share of the batch's rows (all problems run at
+      // once): at least 8, at most the single-problem wave
+      const double share = (double)b->states[i].n[0] / rows_all;
+      int cap = (int)(share * 3.0 * ctx->num_sms + 0.5);
+      c.tsqr_leaf_cap = cap < 8 ? 8 : cap;
+      ttk::Bump dry{nullptr, 0, 0, true};
+      tt_status st = step_dispatch(&c, b->plans[i], &b->states[i], b->tol[i], b->rmax[i], prec, dry);
+      if (st != TT_OK) {
+        ttk::g_instr = prev;
+        release(b);
+        return st;
+      }
+      b->ws_off[i] = total;
+      b->ws_len[i] = dry.need();
+      total += (dry.need() + 255) & ~(size_t)255;
     }
-    b->ws_off[i] = total;
-    b->ws_len[i] = dry.off;
-    total += (dry.off + 255) & ~(size_t)255;
+    if (cudaMalloc(&b->ws, total > 0 ? total : 256) != cudaSuccess) {
+      b->ws = nullptr;
+      (void)cudaGetLastError();
+    }
   }
   ttk::g_instr = prev;
-  if (cudaMalloc(&b->ws, total > 0 ? total : 256) != cudaSuccess) { release(b); return TT_ERR_CUDA; }
+  if (!b->ws) { release(b); return TT_ERR_CUDA; }
   for (int i = 0; i < nprob; ++i) {
     b->sub[i].ws = static_cast<char*>(b->ws) + b->ws_off[i];
     b->sub[i].ws_bytes = b->ws_len[i];

@@ -11,13 +11,18 @@ struct Bump {
   size_t off;
   size_t cap;
   bool dry;
+  size_t peak = 0;  // most that was taken at once (release)
   template <typename T>
   T* take(size_t count) {
     size_t bytes = ((sizeof(T) * (count ? count : 1)) + 255) & ~(size_t)255;
     char* p = dry ? nullptr : base + off;
     off += bytes;
+    if (off > peak) peak = off;
     return reinterpret_cast<T*>(p);
   }
+  // give back everything taken since off was `mark`: later work on the same stream may reuse it
+  void release(size_t mark) { off = mark; }
+  size_t need() const { return off > peak ? off : peak; }
   bool ok() const { return dry || off <= cap; }
 };
 

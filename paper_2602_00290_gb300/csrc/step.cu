@@ -14,6 +14,7 @@
 #include "tsqr_blk.cuh"
 #include "tsqr_rs.cuh"
 #include "tune.cuh"
+#include "xgram.cuh"
 
 namespace ttk {
 namespace {
@@ -290,6 +291,20 @@ inline tt_status run_tsqr_cfg(const TsqrCfg& cfg, cudaStream_t s, int num_sms, c
   return run_tsqr<T, BR>(s, num_sms, src, lp, nrows, cfg.leaves, ws_a, ws_b, Rfinal, leaf_cat);
 }
 
+// Whether a pass takes its triangular factor from the exact Gram products (xgram.cuh): unless the
+// caller chose Householder TSQR kernels for the shape (tt_context_set_tsqr, tt_autotune).
+template <typename T, class Src>
+inline bool xg_takes(const tt_context* ctx, const TsqrCfg& cfg, const Src& src, const LivePattern& lp, long nrows) {
+  return !cfg.set && !ctx->no_xg && xg_fits<T>(src, lp, nrows);
+}
+// SMs such a pass may take: all of them, or a batched problem's share (its leaf cap).
+template <typename T>
+inline int xg_sms(const tt_context* ctx) {
+  if (ctx->tsqr_leaf_cap <= 0) return ctx->num_sms;
+  const int share = (ctx->tsqr_leaf_cap + BigLeaves<T>::per_sm - 1) / BigLeaves<T>::per_sm;
+  return share < ctx->num_sms ? share : ctx->num_sms;
+}
+
 // Workspace carving shared by dry runs (size queries) and real runs.
 struct RoundBufs {
   double* tsqr_a;
@@ -304,10 +319,10 @@ struct RoundBufs {
 };
 
 template <typename T>
-static RoundBufs take_round_bufs(Bump& ws, int num_sms, int max_leaves, int d, int R, long nrows, int n1, int n2,
+static RoundBufs take_round_bufs(Bump& ws, int num_sms, bool tsqr, const TsqrCfg& cfg, int d, int R, long nrows, int n1, int n2,
                                  int K1, int K2, int rcapin1) {
   RoundBufs b;
-  const long L = tsqr_leaf_bound<T>(num_sms, R, nrows, max_leaves);
+  const long L = !tsqr ? 0 : tsqr_leaf_bound<T>(num_sms, R, nrows, cfg.leaves);
   b.tsqr_a = ws.take<double>((size_t)L * R * R);
   b.tsqr_b = ws.take<double>((size_t)((L + 1) / 2) * R * R);
   b.Bbase = ws.take<double>((size_t)rcapin1 * n1 * n2);
@@ -386,7 +401,9 @@ tt_status round_impl(tt_context* ctx, tt_tensor* x, double tol, int rmax, Bump& 
   LivePattern lp{x->rank + 1, K1, 1, 0};
   const int R = lp.ncap();
   const TsqrCfg cfg = tsqr_cfg<T>(ctx, R);
-  RoundBufs b = take_round_bufs<T>(ws, ctx->num_sms, cfg.leaves, d, R, N, n1, n2, K1, K2, K1);
+  const SrcRows<S> src{(const S*)x->core[0], K1};
+  const bool xg = xg_takes<T>(ctx, cfg, src, lp, N);
+  RoundBufs b = take_round_bufs<T>(ws, ctx->num_sms, !xg, cfg, d, R, N, n1, n2, K1, K2, K1);
   SmallJob job{};
   job.d = d;
   job.n1 = n1;
@@ -425,6 +442,9 @@ tt_status round_impl(tt_context* ctx, tt_tensor* x, double tol, int rmax, Bump& 
     tt_status st = randomized_factor<S, T>(ctx, s, SrcRows<S>{(const S*)x->core[0], K1}, lp, N, b.Bbase, n1 * n2, ws,
                                            &RZ, kTsqrLeaf);
     if (st != TT_OK) return st;
+  } else if (xg) {
+    tt_status st = xg_factor<T>(s, ctx->num_sms, xg_sms<T>(ctx), src, lp, N, ws, &RZ, &ctx->ctrl->status);
+    if (st != TT_OK) return st;
   } else if (!ws.dry) {
     tt_status st = run_tsqr_cfg<T>(cfg, s, ctx->num_sms, SrcRows<S>{(const S*)x->core[0], K1}, lp, N, b.tsqr_a,
                                    b.tsqr_b, &RZ);
@@ -455,7 +475,10 @@ tt_status step_impl(tt_context* ctx, const tt_plan* p, tt_tensor* I, double tol,
   LivePattern lp1{I->rank + 1, K1, p->nterm + 1, p->nbc};
   const int R1 = lp1.ncap();
   const TsqrCfg cfg1 = tsqr_cfg<T>(ctx, R1);
-  RoundBufs b1 = take_round_bufs<T>(ws, ctx->num_sms, cfg1.leaves, d, R1, N, n1, n2, K1, K2, K1);
+  SrcStencil<S> src1{};
+  fill_stencil<S>(src1, p, (const S*)I->core[0], K1);
+  const bool xg1 = xg_takes<T>(ctx, cfg1, src1, lp1, N);
+  RoundBufs b1 = take_round_bufs<T>(ws, ctx->num_sms, !xg1, cfg1, d, R1, N, n1, n2, K1, K2, K1);
   S* Zsrc = ws.take<S>((size_t)N * (K1 + 1));
   const long ngrid = (N + 31) / 32;  // bounds the persistent update grids (tiles of >= 32 rows)
   double* part1 = ws.take<double>((size_t)2 * ngrid);
@@ -464,8 +487,6 @@ tt_status step_impl(tt_context* ctx, const tt_plan* p, tt_tensor* I, double tol,
   double* part0 = ws.take<double>((size_t)((N + 255) / 256));
   double* sums = ws.take<double>(8);
   double* vJ0 = ws.take<double>(K1);
-  SrcStencil<S> src1{};
-  fill_stencil<S>(src1, p, (const S*)I->core[0], K1);
   SmallJob j1{};
   j1.d = d;
   j1.n1 = n1;
@@ -509,6 +530,10 @@ tt_status step_impl(tt_context* ctx, const tt_plan* p, tt_tensor* I, double tol,
   } else if (rnd) {
     tt_status st = randomized_factor<S, T>(ctx, s, src1, lp1, N, b1.B0, nang, ws, &RZ1, kTsqrLeaf);
     if (st != TT_OK) return st;
+  } else if (xg1) {
+    tt_status st =
+        xg_factor<T>(s, ctx->num_sms, xg_sms<T>(ctx), src1, lp1, N, ws, &RZ1, &ctx->ctrl->status);
+    if (st != TT_OK) return st;
   } else if (!ws.dry) {
     tt_status st = run_tsqr_cfg<T>(cfg1, s, ctx->num_sms, src1, lp1, N, b1.tsqr_a, b1.tsqr_b, &RZ1);
     if (st != TT_OK) return st;
@@ -519,7 +544,8 @@ tt_status step_impl(tt_context* ctx, const tt_plan* p, tt_tensor* I, double tol,
   // ---- source step fused into the write of the rounded transport update
   LivePattern lp2{nullptr, K1, 1, 1};
   const TsqrCfg cfg2 = tsqr_cfg<T>(ctx, lp2.ncap());
-  RoundBufs b2 = take_round_bufs<T>(ws, ctx->num_sms, cfg2.leaves, d, lp2.ncap(), N, n1, n2, K1, K2, K1);
+  const bool xg2 = xg_takes<T>(ctx, cfg2, SrcRows<S>{Zsrc, K1 + 1}, lp2, N);
+  RoundBufs b2 = take_round_bufs<T>(ws, ctx->num_sms, !xg2, cfg2, d, lp2.ncap(), N, n1, n2, K1, K2, K1);
   double *cpl_u = nullptr, *jstar = nullptr, *jnew = nullptr;
   if (p->coupled) {
     cpl_u = ws.take<double>(R1);
@@ -536,6 +562,11 @@ tt_status step_impl(tt_context* ctx, const tt_plan* p, tt_tensor* I, double tol,
     } else if (rnd) {
       double* RZ2 = nullptr;
       st = randomized_factor<S, T>(ctx, s, SrcRows<S>{Zsrc, K1 + 1}, lp2, N, b2.B0, nang, ws, &RZ2, kTsqrLeafSrc);
+      if (st != TT_OK) return st;
+    } else if (xg2) {
+      double* RZ2 = nullptr;
+      st = xg_factor<T>(s, ctx->num_sms, xg_sms<T>(ctx), SrcRows<S>{Zsrc, K1 + 1}, lp2, N, ws, &RZ2,
+                        &ctx->ctrl->status, kTsqrLeafSrc);
       if (st != TT_OK) return st;
     }
     return small_round(s, ctx->num_sms, j2, ws);
@@ -563,6 +594,9 @@ tt_status step_impl(tt_context* ctx, const tt_plan* p, tt_tensor* I, double tol,
                      kTsqrLeafSrc);
   else if (rnd)
     st = randomized_factor<S, T>(ctx, s, SrcRows<S>{Zsrc, K1 + 1}, lp2, N, b2.B0, nang, ws, &RZ2, kTsqrLeafSrc);
+  else if (xg2)
+    st = xg_factor<T>(s, ctx->num_sms, xg_sms<T>(ctx), SrcRows<S>{Zsrc, K1 + 1}, lp2, N, ws, &RZ2,
+                      &ctx->ctrl->status, kTsqrLeafSrc);
   else
     st = run_tsqr_cfg<T>(cfg2, s, ctx->num_sms, SrcRows<S>{Zsrc, K1 + 1}, lp2, N, b2.tsqr_a, b2.tsqr_b, &RZ2,
                          kTsqrLeafSrc);

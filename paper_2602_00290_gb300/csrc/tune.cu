@@ -150,7 +150,7 @@ tt_status tt_autotune(tt_context* ctx, const tt_plan* plan, const tt_tensor* I, 
       ++tab->epoch;
       if (ttk::resolve_tsqr(ctx, es, ncaps[role], wave).variant != v) continue;  // shape not taken by v
       for (int l : leaf_opts(v)) {
-        if (v == ttk::kTsqrColumn && l == wave) continue;  // the default, timed as `base`
+        if (v == ttk::kTsqrColumn && l == wave) continue;  // reported for the default, timed as `base`
         tab->m[key] = ttk::TsqrCfg{v, l};
         ++tab->epoch;
         float t = 0.0f;
@@ -163,7 +163,11 @@ tt_status tt_autotune(tt_context* ctx, const tt_plan* plan, const tt_tensor* I, 
         }
       }
     }
-    tab->m[key] = ttk::TsqrCfg{pick[role][0], pick[role][1]};
+    // the default (the exact Gram factor, timed as `base`) is kept by leaving the shape without an entry
+    if (pick[role][0] == ttk::kTsqrColumn && pick[role][1] == wave)
+      tab->m.erase(key);
+    else
+      tab->m[key] = ttk::TsqrCfg{pick[role][0], pick[role][1]};
     ++tab->epoch;
   }
   cudaEventDestroy(e0);

@@ -25,6 +25,7 @@ constexpr int kTsqrMaxLeavesPerSm = 6;
 struct TsqrCfg {
   int variant;
   int leaves;  // cap on the leaves; 0: one wave of resident CTAs
+  bool set = false;  // an entry was set (or autotuned) for this shape
 };
 
 struct TsqrTune {
@@ -49,7 +50,7 @@ inline TsqrTune* tune_of(const tt_context* ctx) { return static_cast<TsqrTune*>(
 inline TsqrCfg resolve_tsqr(const tt_context* ctx, int esize, int ncap, int wave) {
   TsqrCfg cfg{kTsqrColumn, 0};
   const TsqrTune* tab = tune_of(ctx);
-  if (tab) tab->find(esize, ncap, &cfg);
+  if (tab) cfg.set = tab->find(esize, ncap, &cfg);
   const int most = kTsqrMaxLeavesPerSm * ctx->num_sms;
   if (ctx->tsqr_leaf_cap > 0 || cfg.leaves <= 0) cfg.leaves = wave;
   else if (cfg.leaves > most) cfg.leaves = most;
