@@ -17,9 +17,12 @@
 // normalised converged columns are the right singular vectors).
 #include <cstddef>
 #include <cstdio>
+#include <type_traits>
 
 #include "bigpass.cuh"
+#include "jacobi_cl.cuh"
 #include "small.cuh"
+#include "xgram.cuh"
 
 namespace ttk {
 namespace {
@@ -926,13 +929,14 @@ __global__ void __launch_bounds__(256) k_permute_cols(int nv, int ldv, int K, co
   }
 }
 
-// Energy beyond the first K of n sorted singular values that are accurate to FP64 (the squared
-// tail, like k_tail_from_parts, but without the cancellation of ||A||^2 - sum sigma^2).
-__global__ void k_tail_from_sigma(int n, int K, const double* __restrict__ sig, double* __restrict__ tail) {
-  if (threadIdx.x || blockIdx.x) return;
+// Energy beyond the K largest of n singular values that are accurate to FP64 (perm: their order; the
+// squared tail, like k_tail_from_parts, but without the cancellation of ||A||^2 - sum sigma^2).  One warp.
+__global__ void k_tail_from_sigma(int n, int K, const double* __restrict__ sig, const int* __restrict__ perm,
+                                  double* __restrict__ tail) {
   double s2 = 0.0;
-  for (int j = n - 1; j >= K; --j) s2 += sig[j] * sig[j];
-  *tail = s2;
+  for (int j = K + (int)threadIdx.x; j < n; j += 32) s2 += sig[perm[j]] * sig[perm[j]];
+  s2 = warp_sum(s2);
+  if (threadIdx.x == 0) *tail = s2;
 }
 
 // Columns j < k of V (nv x ldv, row-major) whose singular value is exactly zero carry no
@@ -2045,9 +2049,29 @@ static tt_status svd_right_f64pre(cudaStream_t s, int num_sms, const Src& src, l
   return cudaGetLastError() == cudaSuccess ? TT_OK : TT_ERR_CUDA;
 }
 
+// The default form of both: the triangular factor from exact Gram products (xgram.cuh: rows graded by
+// pivoting) and the cluster Jacobi on it, FP32 rotations or FP64.
+template <bool F64, class Src>
+static tt_status svd_right_xg(cudaStream_t s, int num_sms, const Src& src, long rows, int cols, Bump& ws,
+                              double** U_out, double** P_out, double* raw, int* perm, DevCtrl* ctrl) {
+  using T = typename std::conditional<F64, double, float>::type;
+  double* U = ws.take<double>((size_t)cols * cols);
+  if (P_out) *P_out = ws.take<double>((size_t)rows * cols);
+  *U_out = U;
+  double* R = nullptr;
+  const tt_status st =
+      xg_factor<T>(s, num_sms, num_sms, src, LivePattern{nullptr, cols, 1, 0}, rows, ws, &R, &ctrl->status);
+  if (st != TT_OK || ws.dry) return st;
+  return launch_jacobi_cl<T>(s, cols, R, U, raw, perm, ctrl);
+}
+
 template <bool F64, class Src>
 static tt_status svd_right_pre(cudaStream_t s, int num_sms, const Src& src, long rows, int cols, Bump& ws,
-                               double** U_out, double** P_out, double* raw, int* perm, DevCtrl* ctrl, int grid_max) {
+                               double** U_out, double** P_out, double* raw, int* perm, DevCtrl* ctrl, int grid_max,
+                               bool xg) {
+  using T = typename std::conditional<F64, double, float>::type;
+  if (xg && cols <= kJcMaxN && xg_fits<T>(src, LivePattern{nullptr, cols, 1, 0}, rows))
+    return svd_right_xg<F64>(s, num_sms, src, rows, cols, ws, U_out, P_out, raw, perm, ctrl);
   if (F64) return svd_right_f64pre(s, num_sms, src, rows, cols, ws, U_out, P_out, raw, perm, ctrl, grid_max);
   return svd_right_mixed(s, num_sms, src, rows, cols, ws, U_out, P_out, raw, perm, ctrl);
 }
@@ -2071,7 +2095,7 @@ static tt_status small_round_mixed3(cudaStream_t s, int num_sms, const SmallJob&
   double* tmp2 = ws.take<double>((size_t)n2 * n2);
   double *U2 = nullptr, *P2 = nullptr;
   tt_status st = svd_right_pre<F64>(s, num_sms, SrcRows<double>{Y, n2}, (long)R * n1, n2, ws, &U2, &P2, sigc2,
-                                   perm2, j.ctrl, j.coop_grid_max);
+                                   perm2, j.ctrl, j.coop_grid_max, !j.no_xg);
   if (st != TT_OK) return st;
   double* P2s = ws.take<double>((size_t)R * n1 * n2);
   const int nv = n1 * K2;
@@ -2119,7 +2143,7 @@ static tt_status small_round_mixed3(cudaStream_t s, int num_sms, const SmallJob&
   double* wpart = ws.take<double>(small_gemm_ksplit_elems(R, K1));
   double *U1 = nullptr, *P1 = nullptr;
   st = svd_right_pre<F64>(s, num_sms, SrcCols<double>{Y2, nv}, nv, R, ws, &U1, &P1, sigc1, perm1, j.ctrl,
-                          j.coop_grid_max);
+                          j.coop_grid_max, !j.no_xg);
   if (st != TT_OK) return st;
   if (!ws.dry) {
     small_gemm<double, double>(s, nv, R, R, Y2, 1, nv, U1, R, 1, P1, R, nullptr, nullptr);  // P1 = A1 U1
@@ -2131,7 +2155,7 @@ static tt_status small_round_mixed3(cudaStream_t s, int num_sms, const SmallJob&
   // energy beyond the Kr refined values: from the FP64 Jacobi singular values (FP64 path), or
   // ||A1||_F^2 - sum sigma_j^2 (mixed path; accurate to about sqrt(eps_64) ||A1||)
   if (F64) {  // the FP64 Jacobi singular values resolve the whole tail
-    k_tail_from_sigma<<<1, 32, 0, s>>>(R, Kr, sigc1, tailK); count_launch();
+    k_tail_from_sigma<<<1, 32, 0, s>>>(R, Kr, sigc1, perm1, tailK); count_launch();
   } else {
     if (few_launches) {
       k_sumsq_parts<<<1, 1024, 0, s>>>((long)R * nv, Y2, nullptr, Kr, sig1, fro1, tailK); count_launch();
@@ -2168,9 +2192,18 @@ tt_status small_round(cudaStream_t s, int num_sms, const SmallJob& j, Bump& ws) 
   if (j.d == 2) {
     // the only bond: SVD of Y (R x n1)
     double* sig = ws.take<double>(n1);
-    double* V = ws.take<double>((size_t)n1 * n1);
-    st = svd_right(s, num_sms, R, n1, Y, ws, sig, V, j.ctrl, j.coop_grid_max);
-    if (st != TT_OK || ws.dry) return st;
+    double* V = nullptr;
+    if (!j.no_xg && n1 <= kJcMaxN && xg_fits<double>(SrcRows<double>{Y, n1}, LivePattern{nullptr, n1, 1, 0}, R)) {
+      int* perm = ws.take<int>(n1);
+      double* tmp = ws.take<double>((size_t)n1 * n1);
+      st = svd_right_xg<true>(s, num_sms, SrcRows<double>{Y, n1}, R, n1, ws, &V, nullptr, sig, perm, j.ctrl);
+      if (st != TT_OK || ws.dry) return st;
+      k_sort_cols<<<1, 1024, 0, s>>>(n1, n1, n1, sig, V, tmp); count_launch();
+    } else {
+      V = ws.take<double>((size_t)n1 * n1);
+      st = svd_right(s, num_sms, R, n1, Y, ws, sig, V, j.ctrl, j.coop_grid_max);
+      if (st != TT_OK || ws.dry) return st;
+    }
     k_decide<<<1, 32, 0, s>>>(sig, n1, 1, 2, j.tol, j.rmax, j.K1cap, j.nrowsZ, j.lp.r_ptr, j.lp.nblk,
                               j.lp.nextra, 1, nullptr, 0, 0, nullptr, 0, n1, j.ctrl, 0, nullptr); count_launch();
     small_gemm<double, double>(s, R, j.K1cap, n1, j.B0, n1, 1, V, n1, 1, j.W, j.K1cap, &j.ctrl->k[0], nullptr);

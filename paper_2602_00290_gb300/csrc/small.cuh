@@ -48,6 +48,7 @@ struct SmallJob {
   double* Bnew;       // [K1cap][n1*n2]
   double* vJ;         // [K1cap]
   DevCtrl* ctrl;      // ranks -> ctrl->k[0] (bond 1), ctrl->k[1] (bond 2)
+  bool no_xg;         // Householder factors and the earlier Jacobi kernels (tt_context::no_xg)
   bool mixed;         // FP32 rotations (Jacobi on R^T of an FP32 TSQR), FP64 singular values/vectors
 };
 

@@ -426,6 +426,7 @@ tt_status round_impl(tt_context* ctx, tt_tensor* x, double tol, int rmax, Bump& 
   job.vJ = b.vJ;
   job.ctrl = ctx->ctrl;
   job.coop_grid_max = ctx->coop_grid_max;
+  job.no_xg = ctx->no_xg != 0;
   job.mixed = (sizeof(T) == 4);
   double* domega_ones = ws.take<double>((size_t)n1 * n2);
   job.domega = domega_ones;
@@ -509,6 +510,7 @@ tt_status step_impl(tt_context* ctx, const tt_plan* p, tt_tensor* I, double tol,
   j1.vJ = b1.vJ;
   j1.ctrl = ctx->ctrl;
   j1.coop_grid_max = ctx->coop_grid_max;
+  j1.no_xg = ctx->no_xg != 0;
   j1.mixed = (sizeof(T) == 4);
   double* RZ1 = nullptr;
   if (!ws.dry) {

@@ -60,6 +60,7 @@ struct XgArray {
   int ncol, G, oc;  // columns, rows per cell, octets per cell
   long ncell;
   int rec;          // bytes of an octet's record
+  long sr, sc;      // element strides of rows and columns
 };
 
 // One column group of the products: `w` columns (a multiple of 8, the last ones padding) of an array, at
@@ -273,10 +274,10 @@ __device__ __forceinline__ void xg_digits2(long long v0, long long v1, unsigned 
 }
 
 // Column maxima |x| (as FP64 bit patterns, over the finite entries: Inf and NaN are latched where the
-// rows are rewritten) of a row-major matrix of ncol <= 256 columns: a CTA takes whole rows, a thread
-// always the same column, eight loads in flight.
+// rows are rewritten) of a matrix of ncol <= 256 columns: a CTA takes whole rows, a thread always the
+// same column, eight loads in flight.
 template <typename S>
-__global__ void __launch_bounds__(256) k_xg_colmax(const S* __restrict__ A, int ncol, long nrows,
+__global__ void __launch_bounds__(256) k_xg_colmax(const S* __restrict__ A, int ncol, long sr, long sc, long nrows,
                                                    unsigned long long* __restrict__ slots,
                                                    const double* __restrict__ bc, int nbc, int G) {
   __shared__ unsigned long long sm[256];
@@ -292,7 +293,7 @@ __global__ void __launch_bounds__(256) k_xg_colmax(const S* __restrict__ A, int 
     for (; k + 7 * step < nrows; k += 8 * step) {
       S v[8];
 #pragma unroll
-      for (int u = 0; u < 8; ++u) v[u] = A[(k + u * step) * ncol + col];
+      for (int u = 0; u < 8; ++u) v[u] = A[(k + u * step) * sr + col * sc];
 #pragma unroll
       for (int u = 0; u < 8; ++u) {
         const S a = fabs(v[u]);
@@ -300,7 +301,7 @@ __global__ void __launch_bounds__(256) k_xg_colmax(const S* __restrict__ A, int 
       }
     }
     for (; k < nrows; k += step) {
-      const S a = fabs(A[k * ncol + col]);
+      const S a = fabs(A[k * sr + col * sc]);
       m = (a > m && a <= kMax) ? a : m;
     }
     atomicMax(&sm[col], (unsigned long long)__double_as_longlong((double)m));
@@ -338,7 +339,7 @@ __global__ void __launch_bounds__(256) k_xg_digits(const S* __restrict__ A, XgAr
     const bool ok = c < ar.ncol && lp.live(c, r);
     S x[8];
 #pragma unroll
-    for (int u = 0; u < 8; ++u) x[u] = (ok && g0 + u < ar.G && k0 + u < nrows) ? A[(k0 + u) * ar.ncol + c] : S(0);
+    for (int u = 0; u < 8; ++u) x[u] = (ok && g0 + u < ar.G && k0 + u < nrows) ? A[(k0 + u) * ar.sr + c * ar.sc] : S(0);
     const int K = xg_shift_const(S(0), ok ? xg_unit(slots[c], NS) : 0);
     unsigned dig[4][NS];
 #pragma unroll
@@ -748,8 +749,8 @@ __device__ __forceinline__ XgComb xg_comb(const SrcStencil<S>& s, int c) {
   else { put(Hh, 1); put(C, -1); }
   return x;
 }
-template <typename S>
-__device__ __forceinline__ XgComb xg_comb(const SrcRows<S>&, int c) {
+template <class Src>
+__device__ __forceinline__ XgComb xg_comb(const Src&, int c) {
   return XgComb{1, {c, 0, 0}, {1, 0, 0}, c, 1.0};
 }
 
@@ -811,6 +812,8 @@ struct XgElem;
 template <typename S>
 struct XgElem<SrcRows<S>> { using type = S; };
 template <typename S>
+struct XgElem<SrcCols<S>> { using type = S; };
+template <typename S>
 struct XgElem<SrcStencil<S>> { using type = S; };
 
 // Plan of a source's columns.
@@ -820,6 +823,10 @@ inline bool xg_make_plan(const SrcRows<S>&, const LivePattern& lp, XgPlan& pl) {
   pl.nsub = 0;
   pl.nraw = n;
   return n <= kXcMaxN && xg_add<NS>(pl, n, 0, 0, 0) && xg_tiles<NS>(pl, false) && xg_stages(pl) >= 2;
+}
+template <int NS, typename S>
+inline bool xg_make_plan(const SrcCols<S>&, const LivePattern& lp, XgPlan& pl) {
+  return xg_make_plan<NS>(SrcRows<S>{nullptr, 0}, lp, pl);
 }
 template <int NS, typename S>
 inline bool xg_make_plan(const SrcStencil<S>& s, const LivePattern& lp, XgPlan& pl) {
@@ -835,24 +842,31 @@ inline bool xg_make_plan(const SrcStencil<S>& s, const LivePattern& lp, XgPlan& 
 }
 template <typename S>
 inline bool xg_array(const SrcRows<S>& s, int n, long nrows, int NS, XgArray& ar, const S** A) {
-  ar = XgArray{n, 8, 1, (nrows + 7) / 8, NS == 4 ? xg_record<4>(n) : xg_record<7>(n)};
+  ar = XgArray{n, 8, 1, (nrows + 7) / 8, NS == 4 ? xg_record<4>(n) : xg_record<7>(n), s.ld, 1};
   *A = s.A;
-  return s.ld == n && ar.ncell < (1L << 31);
+  return ar.ncell < (1L << 31);
+}
+template <typename S>
+inline bool xg_array(const SrcCols<S>& s, int n, long nrows, int NS, XgArray& ar, const S** A) {
+  ar = XgArray{n, 8, 1, (nrows + 7) / 8, NS == 4 ? xg_record<4>(n) : xg_record<7>(n), 1, s.ld};
+  *A = s.A;
+  return ar.ncell < (1L << 31);
 }
 template <typename S>
 inline bool xg_array(const SrcStencil<S>& s, int, long nrows, int NS, XgArray& ar, const S** A) {
-  ar = XgArray{s.rcap, s.G, (s.G + 7) / 8, nrows / s.G, NS == 4 ? xg_record<4>(s.rcap) : xg_record<7>(s.rcap)};
+  ar = XgArray{s.rcap, s.G, (s.G + 7) / 8, nrows / s.G, NS == 4 ? xg_record<4>(s.rcap) : xg_record<7>(s.rcap),
+               s.ldz, 1};
   *A = s.Z;
-  return s.ldz == s.rcap && ar.ncell * ar.oc < (1L << 31);
+  return ar.ncell * ar.oc < (1L << 31);
 }
-template <typename S>
-inline LivePattern xg_array_live(const SrcRows<S>&, const LivePattern& lp) { return lp; }
+template <class Src>
+inline LivePattern xg_array_live(const Src&, const LivePattern& lp) { return lp; }
 template <typename S>
 inline LivePattern xg_array_live(const SrcStencil<S>&, const LivePattern& lp) {
   return LivePattern{lp.r_ptr, lp.rcap, 1, 0};
 }
-template <typename S>
-inline void xg_geometry(const SrcRows<S>&, XgArgs& a, const double** bc, int*) {
+template <class Src>
+inline void xg_geometry(const Src&, XgArgs& a, const double** bc, int*) {
   a.nax = 0;
   *bc = nullptr;
 }
@@ -869,8 +883,8 @@ inline void xg_geometry(const SrcStencil<S>& s, XgArgs& a, const double** bc, in
 
 // The plan of a source's columns, kept per shape and host thread (a pure function of the shape: the
 // greedy assignment takes some microseconds, and a step asks several times).
-template <typename S>
-inline long xg_plan_key(const SrcRows<S>&, const LivePattern& lp) { return lp.ncap(); }
+template <class Src>
+inline long xg_plan_key(const Src&, const LivePattern& lp) { return lp.ncap(); }
 template <typename S>
 inline long xg_plan_key(const SrcStencil<S>& s, const LivePattern& lp) {
   return 1000000L * (1 + s.nax) + 1000L * s.rcap + 10L * lp.nextra + 100000000L * lp.nblk;
@@ -925,7 +939,7 @@ void xg_launch_digits(cudaStream_t s, int num_sms, const S* A, const XgArray& ar
                       unsigned long long* slots, unsigned char* dig, const double* bc, int nbc, unsigned char* bcdig) {
   const long rpb = 256 / ar.ncol, need = (nrows + 8 * rpb - 1) / (8 * rpb);
   long grid = need < 8L * num_sms ? need : 8L * num_sms;
-  k_xg_colmax<S><<<(unsigned)(grid > 0 ? grid : 1), 256, 0, s>>>(A, ar.ncol, nrows, slots, bc, nbc, ar.G);
+  k_xg_colmax<S><<<(unsigned)(grid > 0 ? grid : 1), 256, 0, s>>>(A, ar.ncol, ar.sr, ar.sc, nrows, slots, bc, nbc, ar.G);
   count_launch();
   const long tot = ar.ncell * ar.oc * (ar.rec / (NS * 16));
   grid = (tot + 255) / 256;
