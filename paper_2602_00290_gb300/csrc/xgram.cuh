@@ -2,14 +2,14 @@
 // merged core's columns from them (the L->R orthogonalisation of the rounding, Sec. 3.1 footnote).
 //
 // Every storage column c is held in fixed point, v = round(x 2^-U_c) with one power of two per column,
-// and v is written in balanced digits of base 512,
-//   v = sum_j d_j 512^(NS-1-j),   -256 <= d_j <= 255,
-// NS = 4 digits (34 bits and sign) for FP32 passes and NS = 7 (61 bits and sign) for FP64 passes.
-// Digits are exact in FP16, products of two digits are integers up to 2^16, and the FP32
+// and v is written in balanced digits of base 256,
+//   v = sum_j d_j 256^(NS-1-j),   -128 <= d_j <= 127,
+// NS = 4 digits (30 bits and sign) for FP32 passes and NS = 8 (62 bits and sign) for FP64 passes.
+// Digits are exact in FP16, products of two digits are integers up to 2^14, and the FP32
 // accumulators of tcgen05.mma.kind::f16 sum 256 rows of them without any rounding (every partial sum is
-// an integer of at most 2^24).  The digit products of a chunk are then folded into 64-bit integers.
+// an integer of at most 2^22).  The digit products of a chunk are then folded into 64-bit integers.
 // So sum_k v_a v_b comes out exactly, for columns whose entries carry a fixed-point rounding of at most
-// 2^-(9 NS - 1) of their column's largest entry (FP32 2^-35, FP64 2^-62; the storage's own rounding of
+// 2^-(8 NS - 1) of their column's largest entry (FP32 2^-31, FP64 2^-63; the storage's own rounding of
 // entries near that size is 2^-25 and 2^-54).  The columns of the transport sum are integer
 // combinations of a row and its neighbours (C - L, H - C, H - L, H - 2 C + L), so their Gram matrix is an
 // integer combination of the products of the neighbour blocks, formed without rounding or
@@ -24,10 +24,12 @@
 // columns are written once (k_xg_digits, bound by memory) in the layout of the MMA operands, so that the
 // product kernel (k_xg_mma) only moves 16-byte rows with bulk copies: a neighbour block is the same
 // digits at another cell, a missing neighbour a page of zeros.  Measured for both roundings of a step
-// at 1,048,576 rows, rank 32: FP32 digits 0.19, products 0.87, Cholesky 0.41 ms (leaves and merges before:
-// 6.0 + 2.1 ms); FP64 0.25, 3.06, 0.41 ms (before 99.6 + 14 ms).
+// at 1,048,576 rows, rank 32: FP32 digits 0.18, products 0.67 ms (leaves and merges before: 6.0 + 2.1 ms);
+// FP64 0.28, 1.8 ms (before 99.6 + 14 ms).  With base 512 and MMAs of N = 128 columns over octets copied one by
+// one the products took 0.87 and 3.06 ms.
 #pragma once
 #include <map>
+#include <vector>
 
 #include "bigpass.cuh"
 #include "instr.cuh"
@@ -38,30 +40,39 @@
 namespace ttk {
 
 constexpr int kXgThreads = 576;   // 16 folding warps, a copying warp, an MMA warp
-constexpr int kXgTiles = 4;       // output tiles a CTA accumulates (TMEM: 4 x 128 columns)
+constexpr int kXgGroups = 2;      // MMA groups of a CTA: one block of rows x up to two blocks (N <= 256)
+constexpr int kXgTiles = 4;       // output tiles of a CTA (TMEM: 4 x 128 columns)
+constexpr int kXgChunkTiles = 16; // tiles of 64 rows between two folds: 1024 * 2^14 = 2^24 is exact
 constexpr int kXgMaxBlk = 6;      // operand blocks a CTA stages
 constexpr int kXgMaxSub = 56;     // column groups of a pass
 constexpr int kXgMaxNb = 24;      // operand blocks of a pass
 constexpr int kXgMaxCta = 80;     // CTAs that share a row range
 constexpr int kXgMaxStage = 6;
-constexpr long kXgMaxOct = 2048L * 32;  // row octets per CTA: the 64-bit sums stay below 2^62
+constexpr long kXgMaxPieces = 512L * 16;  // pieces per CTA: at most 512 chunks, the 64-bit sums stay below 2^58
 constexpr int kXgMaxRaw = 448;          // storage columns of all neighbour blocks
 
 template <int NS>
 struct XgCfg {
   static constexpr int W = NS == 4 ? 32 : 16;  // columns per operand block (NS * W <= 128 rows)
-  static constexpr int H = NS == 4 ? 1 : 2;    // 64-bit sums per entry (digit groups of 4 and 3)
+  static constexpr int H = NS / 4;             // 64-bit sums per entry (groups of 4 digits)
 };
 
-// A row-major storage matrix whose rows are the groups of cells (row = g + G cell), or plain rows
-// (G = 8, ncell = ceil(nrows / 8)).  Its digits are kept per octet of rows (a cell's groups padded to a
-// multiple of 8): record = for each column group, for digit j, for column a: eight rows in 16 bytes.
+// A storage matrix whose rows are the groups of cells (row = g + G cell), or plain rows (cells of 64).  Its
+// digits are kept in pieces: a cell's rows (padded) in `parts` pieces of `po` octets, po even and at most
+// 8, so that a piece is a run of K for the MMAs and every neighbour's rows are pieces too.  One plane per
+// column group: [cell][part][rows j w + a of the operand in eights][octet][8 rows x 16 bytes].
 struct XgArray {
-  int ncol, G, oc;  // columns, rows per cell, octets per cell
-  long ncell;
-  int rec;          // bytes of an octet's record
-  long sr, sc;      // element strides of rows and columns
+  int ncol, G, po, parts;
+  long ncell, npiece;  // npiece = ncell * parts
+  int cpad;            // columns with the groups' padding
+  long sr, sc;         // element strides of rows and columns
 };
+inline void xg_pieces(XgArray& ar) {
+  const int oc = (ar.G + 7) / 8;
+  ar.parts = (oc + 7) / 8;
+  ar.po = ((oc + ar.parts - 1) / ar.parts + 1) & ~1;
+  ar.npiece = ar.ncell * ar.parts;
+}
 
 // One column group of the products: `w` columns (a multiple of 8, the last ones padding) of an array, at
 // the cell itself (nb = 0), its lower (1 + 2 axis) or upper (2 + 2 axis) neighbour, or the inflow column
@@ -69,27 +80,28 @@ struct XgArray {
 struct XgSub {
   short raw0;        // first raw column
   unsigned char cnt, w, arr, nb;
-  int off;           // byte offset in the array's record
+  int c0;            // columns (with padding) in the planes before
 };
 
 struct XgPlan {
-  int ns, nsub, nb, ncta, ntile, nraw;
+  int ns, nsub, nb, ncta, nraw;
   XgSub sub[kXgMaxSub];
   unsigned char bsub0[kXgMaxNb], bnsub[kXgMaxNb];  // operand block -> its column groups (equal widths)
-  unsigned char ctiles[kXgMaxCta], cblks[kXgMaxCta];
-  unsigned char tp[kXgMaxCta][kXgTiles], tq[kXgMaxCta][kXgTiles];  // tile -> local block of p, q
-  unsigned char blk[kXgMaxCta][kXgMaxBlk];                         // local block -> operand block
-  short tile0[kXgMaxCta];                                          // first tile of the CTA
-  unsigned char gp[kXgMaxCta * kXgTiles], gq[kXgMaxCta * kXgTiles];
+  unsigned char cgroups[kXgMaxCta], cblks[kXgMaxCta];
+  unsigned char blk[kXgMaxCta][kXgMaxBlk];           // local block -> operand block, in the stage's order
+  unsigned char gm[kXgMaxCta][kXgGroups];            // MMA group: local block of the rows,
+  unsigned char gn[kXgMaxCta][kXgGroups], gnn[kXgMaxCta][kXgGroups];  // first local block of the columns, and how many
+  unsigned char tp[kXgMaxCta * kXgTiles], tq[kXgMaxCta * kXgTiles];   // tile 4 cta + 2 group + h: blocks (p, q);
+                                                                      // p = 255: unused
 };
 
 // What the product kernel reads beside the plan.
 struct XgArgs {
   const unsigned char* dig[2];  // digit records of the arrays
-  const unsigned char* bc;      // digit records of one cell of the inflow columns: [face slot][octet]
+  const unsigned char* bc;      // digit pieces of one cell of the inflow columns: [face slot][part]
   const unsigned char* zero;    // a page of zeros
-  int oc, rec[2], bcrec;
-  long noct, opg;               // octets in all, and per row group
+  int po, parts, nc;            // octets of a piece, pieces of a cell, pieces of a stage
+  long npiece, ppg;             // pieces in all, and per row group
   int nax, ext[3];
   int cstr[3];                  // cell strides of the axes
   unsigned char face[6];        // inflow column -> 2 axis + (upper face)
@@ -106,28 +118,23 @@ __host__ __device__ inline int xg_block_rows(const XgPlan& pl, int b) {
 template <int NS>
 inline bool xg_add(XgPlan& pl, int ncol, int raw0, int arr, int nb) {
   constexpr int W = XgCfg<NS>::W;
-  int off = 0;
+  int c0 = 0;
   for (int c = 0; c < ncol; c += W) {
     if (pl.nsub == kXgMaxSub) return false;
     const int cnt = ncol - c < W ? ncol - c : W, w = (cnt + 7) & ~7;
     pl.sub[pl.nsub++] = XgSub{(short)(raw0 + c), (unsigned char)cnt, (unsigned char)w, (unsigned char)arr,
-                              (unsigned char)nb, off};
-    off += NS * w * 16;
+                              (unsigned char)nb, c0};
+    c0 += w;
   }
   return true;
 }
-template <int NS>
-inline int xg_record(int ncol) {
-  constexpr int W = XgCfg<NS>::W;
-  int off = 0;
-  for (int c = 0; c < ncol; c += W) off += NS * (((ncol - c < W ? ncol - c : W) + 7) & ~7) * 16;
-  return off;
-}
 
-// Operand blocks (column groups of one width side by side, at most W columns; with 7 digits always 16, a
-// padding group where one is missing, since an MMA's N is a multiple of 16), and the output tiles of each
-// CTA: the upper triangle of the blocks, or (arrays: split) blocks of array 0 x blocks of array 1.  A CTA
-// takes up to four tiles that share blocks: the next tile is one that adds the fewest.
+// Operand blocks (column groups of one width side by side, at most W columns), and the MMA groups of each
+// CTA: the upper triangle of the blocks, or (arrays: split) blocks of array 0 x blocks of array 1.  A group
+// is one block of rows times an aligned pair of blocks (N = 256: an MMA of N = 128 takes as long as one
+// of 256, measured 1,930 against 1,070 cycles for 16 products of 128 x 128 x 16); an odd last block takes
+// the rows against every pair.  A CTA has two groups (512 TMEM columns), the second one chosen to share
+// most blocks with the first.
 template <int NS>
 inline bool xg_tiles(XgPlan& pl, bool split) {
   constexpr int W = XgCfg<NS>::W;
@@ -142,7 +149,6 @@ inline bool xg_tiles(XgPlan& pl, bool split) {
       int room = 0;
       for (int i = 0; i < n; ++i) {
         if (in[i].w != w || (split && in[i].arr != arr)) continue;
-        if (pl.nsub == kXgMaxSub) return false;
         if (room < w) {
           if (pl.nb == kXgMaxNb) return false;
           pl.bsub0[pl.nb] = (unsigned char)pl.nsub;
@@ -153,58 +159,74 @@ inline bool xg_tiles(XgPlan& pl, bool split) {
         ++pl.bnsub[pl.nb - 1];
         room -= w;
       }
-      if (NS == 7 && w == 8 && room == 8) {
-        if (pl.nsub == kXgMaxSub) return false;
-        pl.sub[pl.nsub++] = XgSub{0, 0, 8, 0, 255, 0};  // padding: zeros
-        ++pl.bnsub[pl.nb - 1];
-      }
     }
     if (arr == 0) nleft = pl.nb;
   }
-  const int q0 = split ? nleft : 0, np = split ? nleft : pl.nb;
-  bool done[kXgMaxNb][kXgMaxNb] = {};
-  int open = 0;
-  for (int p = 0; p < np; ++p)
-    for (int q = (split ? q0 : p); q < pl.nb; ++q) ++open;
-  pl.ncta = pl.ntile = 0;
-  while (open > 0) {
+  struct Group {
+    int m, n0, nn;
+  };
+  std::vector<Group> gr;
+  const int q0 = split ? nleft : 0, np = split ? nleft : pl.nb, nq = pl.nb - q0;
+  if (split) {
+    for (int j = 0; j < nq; j += 2)
+      for (int p = 0; p < np; ++p) gr.push_back({p, q0 + j, j + 1 < nq ? 2 : 1});
+  } else {
+    for (int j = 0; j + 1 < nq; j += 2)
+      for (int p = 0; p <= j + 1; ++p) gr.push_back({p, j, 2});
+    if (nq & 1) {
+      for (int j = 0; j + 1 < nq; j += 2) gr.push_back({nq - 1, j, 2});
+      gr.push_back({nq - 1, nq - 1, 1});
+    }
+  }
+  pl.ncta = 0;
+  while (!gr.empty()) {
     if (pl.ncta == kXgMaxCta) return false;
     const int k = pl.ncta++;
-    int nblk = 0, nt = 0;
-    unsigned char blk[kXgMaxBlk];
-    pl.tile0[k] = (short)pl.ntile;
+    int nblk = 0;
+    unsigned char* blk = pl.blk[k];
     auto local = [&](int b) {
       for (int i = 0; i < nblk; ++i)
         if (blk[i] == b) return i;
       return -1;
     };
-    while (nt < kXgTiles && open > 0) {
-      int bp = -1, bq = -1, best = 3;
-      for (int p = 0; p < np; ++p)
-        for (int q = (split ? q0 : p); q < pl.nb; ++q) {
-          if (done[p][q]) continue;
-          const int add = (local(p) < 0) + (p != q && local(q) < 0);
-          if (add < best) {
-            best = add;
-            bp = p;
-            bq = q;
-          }
-        }
-      if (nblk + best > kXgMaxBlk || (nt > 0 && best == 2)) break;
-      if (local(bp) < 0) blk[nblk++] = (unsigned char)bp;
-      if (local(bq) < 0) blk[nblk++] = (unsigned char)bq;
-      done[bp][bq] = true;
-      --open;
-      pl.tp[k][nt] = (unsigned char)local(bp);
-      pl.tq[k][nt] = (unsigned char)local(bq);
-      pl.gp[pl.ntile] = (unsigned char)bp;
-      pl.gq[pl.ntile] = (unsigned char)bq;
-      ++pl.ntile;
-      ++nt;
+    auto added = [&](const Group& g) {  // blocks a group adds
+      int a = 0;
+      for (int i = 0; i < g.nn; ++i) a += local(g.n0 + i) < 0;
+      return a + (local(g.m) < 0 && (g.m < g.n0 || g.m >= g.n0 + g.nn));
+    };
+    Group mine[kXgGroups];
+    int ng = 0;
+    while (ng < kXgGroups && !gr.empty()) {
+      size_t best = 0;
+      for (size_t i = 1; i < gr.size(); ++i)
+        if (added(gr[i]) < added(gr[best])) best = i;
+      const Group g = gr[best];
+      gr.erase(gr.begin() + best);
+      mine[ng++] = g;
+      // a pair's blocks lie side by side in the stage: aligned pairs are always added whole
+      if (local(g.n0) < 0 || (g.nn == 2 && local(g.n0 + 1) != local(g.n0) + 1))
+        for (int i = 0; i < g.nn; ++i) blk[nblk++] = (unsigned char)(g.n0 + i);
+      if (local(g.m) < 0) blk[nblk++] = (unsigned char)g.m;
     }
-    pl.ctiles[k] = (unsigned char)nt;
+    pl.cgroups[k] = (unsigned char)ng;
     pl.cblks[k] = (unsigned char)nblk;
-    for (int i = 0; i < nblk; ++i) pl.blk[k][i] = blk[i];
+    for (int g = 0; g < kXgGroups; ++g)
+      for (int h = 0; h < 2; ++h) {
+        const int t = kXgTiles * k + 2 * g + h;
+        pl.tp[t] = pl.tq[t] = 255;
+        if (g >= ng || h >= mine[g].nn) continue;
+        const int p = mine[g].m, q = mine[g].n0 + h;
+        // the entry below the diagonal of a diagonal pair, and an odd last block's row against itself
+        // through a pair, have their mirror elsewhere
+        if (!split && p > q && !((nq & 1) && p == nq - 1)) continue;
+        pl.tp[t] = (unsigned char)p;
+        pl.tq[t] = (unsigned char)q;
+      }
+    for (int g = 0; g < ng; ++g) {
+      pl.gm[k][g] = (unsigned char)local(mine[g].m);
+      pl.gn[k][g] = (unsigned char)local(mine[g].n0);
+      pl.gnn[k][g] = (unsigned char)mine[g].nn;
+    }
   }
   return true;
 }
@@ -219,7 +241,7 @@ inline size_t xg_stage_bytes(const XgPlan& pl) {
   }
   return most;
 }
-constexpr size_t kXgPad = 128 * 16;  // an M = 128 operand of a narrower block reads past its last octet
+constexpr size_t kXgPad = 16 * 1024;  // an M = 128 operand of a narrower block reads past its piece
 inline int xg_stages(const XgPlan& pl) {
   const int n = (int)((226 * 1024 - kXgPad) / xg_stage_bytes(pl));
   return n < kXgMaxStage ? n : kXgMaxStage;
@@ -227,9 +249,9 @@ inline int xg_stages(const XgPlan& pl) {
 
 // ---- fixed point ---------------------------------------------------------------------------------
 // Unit exponent U of a column with largest magnitude `maxbits` (an FP64 bit pattern): every entry is
-// below 2^E, and 2^E maps to 2^(9 NS - 2), inside the digits' range.
+// below 2^E, and 2^E maps to 2^(8 NS - 2), inside the digits' range.
 __host__ __device__ inline int xg_unit(unsigned long long maxbits, int NS) {
-  return ((int)((maxbits >> 52) & 0x7ff) - 1022) - (9 * NS - 2);
+  return ((int)((maxbits >> 52) & 0x7ff) - 1022) - (8 * NS - 2);
 }
 // round(x 2^-U), U folded into the shift constant K (see xg_shift_const).  An exponent field of zero
 // (zero, denormals) gives 0; Inf and NaN give some in-range integer.
@@ -237,7 +259,7 @@ __device__ __forceinline__ long long xg_fix(double x, int K) {
   const unsigned long long b = (unsigned long long)__double_as_longlong(x);
   const int e = (int)((b >> 52) & 0x7ff);
   const unsigned long long m = e ? (((b & 0xfffffffffffffull) | 0x10000000000000ull) << 10) : 0ull;
-  const int sh = min(max(K - e, 1), 63);
+  const int sh = min(max(K - e, 0), 63);
   const long long r = (long long)(((m >> sh) + 1ull) >> 1);
   return (long long)b < 0 ? -r : r;
 }
@@ -245,30 +267,26 @@ __device__ __forceinline__ long long xg_fix(float x, int K) {
   const unsigned b = __float_as_uint(x);
   const int e = (int)((b >> 23) & 0xff);
   const unsigned long long m = e ? ((unsigned long long)((b & 0x7fffffu) | 0x800000u) << 39) : 0ull;
-  const int sh = min(max(K - e, 1), 63);
+  const int sh = min(max(K - e, 0), 63);
   const long long r = (long long)(((m >> sh) + 1ull) >> 1);
   return (int)b < 0 ? -r : r;
 }
 __device__ __forceinline__ int xg_shift_const(double, int U) { return 1084 + U; }
 __device__ __forceinline__ int xg_shift_const(float, int U) { return 188 + U; }
 
-// sum of 256 * 512^s over the NS digits: v + bias has the biased digits 0..511
-template <int NS>
-__host__ __device__ constexpr unsigned long long xg_bias() {
-  unsigned long long b = 0;
-  for (int s = 0; s < NS; ++s) b |= 256ull << (9 * s);
-  return b;
-}
-// Digits of two rows of one column packed as FP16 pairs: dig[j] = (row 0, row 1) for digit j.
+// Digits of two rows of one column packed as FP16 pairs: dig[j] = (row 0, row 1) for digit j.  v + bias
+// (128 in every byte) has the biased digits 0..255 as its bytes.
 template <int NS>
 __device__ __forceinline__ void xg_digits2(long long v0, long long v1, unsigned (&dig)[NS]) {
-  const unsigned long long u0 = (unsigned long long)v0 + xg_bias<NS>(), u1 = (unsigned long long)v1 + xg_bias<NS>();
+  constexpr unsigned long long kBias = 0x8080808080808080ull >> (64 - 8 * NS);
+  const unsigned long long u0 = (unsigned long long)v0 + kBias, u1 = (unsigned long long)v1 + kBias;
 #pragma unroll
   for (int j = 0; j < NS; ++j) {
-    const int s = 9 * (NS - 1 - j);
-    const unsigned a = (unsigned)(u0 >> s), b = (unsigned)(u1 >> s);
-    unsigned x = (__byte_perm(a, b, 0x5410) & 0x01ff01ffu) | 0x64006400u;  // 1024 + biased digit
-    asm("sub.rn.f16x2 %0, %0, %1;" : "+r"(x) : "r"(0x65006500u));          // - 1280
+    const int byte = NS - 1 - j;
+    const unsigned a = (unsigned)(u0 >> (32 * (byte / 4))), b = (unsigned)(u1 >> (32 * (byte / 4)));
+    const unsigned k = (unsigned)(byte % 4);
+    unsigned x = (__byte_perm(a, b, k | (4u + k) << 8) & 0x00ff00ffu) | 0x64006400u;  // 1024 + biased digit
+    asm("sub.rn.f16x2 %0, %0, %1;" : "+r"(x) : "r"(0x64806480u));                     // - 1152
     dig[j] = x;
   }
 }
@@ -313,9 +331,15 @@ __global__ void __launch_bounds__(256) k_xg_colmax(const S* __restrict__ A, int 
       atomicMax(&slots[ncol + i / G], (unsigned long long)__double_as_longlong(fabs(bc[i])));
 }
 
-// Digit records of an array (and, in the CTAs past its octets, of the inflow columns: one cell, one
-// column each): a thread forms one column of one octet, eight rows, and writes 16 bytes per digit.
-// Bound by memory: N r (sizeof(S) + 2 NS) bytes.
+// Byte offset of row m's octet in a plane of groups of w columns (NS w rows) at piece `piece`.
+template <int NS>
+__device__ __forceinline__ size_t xg_dig_off(long piece, int po, int w, int m, int oct) {
+  return ((size_t)piece * (NS * w / 8) + (m >> 3)) * (size_t)(po * 128) + oct * 128 + (m & 7) * 16;
+}
+
+// Digits of an array (and, in the first CTA, of the inflow columns: one cell, one column each): a thread
+// forms one column of one octet, eight rows, and writes 16 bytes per digit.  Bound by memory:
+// N r (sizeof(S) + 2 NS) bytes.
 template <int NS, typename S>
 __global__ void __launch_bounds__(256) k_xg_digits(const S* __restrict__ A, XgArray ar, LivePattern lp, long nrows,
                                                    const unsigned long long* __restrict__ slots,
@@ -323,16 +347,18 @@ __global__ void __launch_bounds__(256) k_xg_digits(const S* __restrict__ A, XgAr
                                                    int nbc, unsigned char* __restrict__ bcout) {
   constexpr int W = XgCfg<NS>::W;
   const int r = lp.r_ptr ? *lp.r_ptr : lp.rcap;
-  const int cpad = ar.rec / (NS * 16);  // columns with padding
-  const long noct = ar.ncell * ar.oc;
+  const int cpad = ar.cpad;
+  const long noct = ar.npiece * ar.po;
   const long tot = noct * cpad;
   long i = blockIdx.x * (long)blockDim.x + threadIdx.x;
   for (; i < tot; i += (long)gridDim.x * blockDim.x) {
     const long oct = tot < (1L << 31) ? (long)((unsigned)i / (unsigned)cpad) : i / cpad;
     const int c = (int)(i - oct * cpad);
-    const long cell = (long)((unsigned)oct / (unsigned)ar.oc);
-    const int g0 = (int)(oct - cell * ar.oc) * 8;
-    const long k0 = cell * ar.G + g0;
+    const unsigned piece = (unsigned)oct / (unsigned)ar.po;
+    const int oin = (int)((unsigned)oct - piece * (unsigned)ar.po);
+    const unsigned cell = ar.parts == 1 ? piece : piece / (unsigned)ar.parts;
+    const int g0 = ((int)(piece - cell * (unsigned)ar.parts) * ar.po + oin) * 8;
+    const long k0 = (long)cell * ar.G + g0;
     // column groups are full blocks of W and then the rest: the width of this column's group
     const int blk = c / W, a = c - blk * W;
     const int w = cpad - blk * W < W ? cpad - blk * W : W;
@@ -344,15 +370,17 @@ __global__ void __launch_bounds__(256) k_xg_digits(const S* __restrict__ A, XgAr
     unsigned dig[4][NS];
 #pragma unroll
     for (int u = 0; u < 4; ++u) xg_digits2<NS>(xg_fix(x[2 * u], K), xg_fix(x[2 * u + 1], K), dig[u]);
-    unsigned char* o = out + oct * ar.rec + (size_t)(blk * W * NS) * 16;
+    unsigned char* o = out + (size_t)(blk * W) * noct * (NS * 16);
 #pragma unroll
     for (int j = 0; j < NS; ++j)
-      *reinterpret_cast<uint4*>(o + (j * w + a) * 16) = make_uint4(dig[0][j], dig[1][j], dig[2][j], dig[3][j]);
+      *reinterpret_cast<uint4*>(o + xg_dig_off<NS>(piece, ar.po, w, j * w + a, oin)) =
+          make_uint4(dig[0][j], dig[1][j], dig[2][j], dig[3][j]);
   }
   if (blockIdx.x == 0 && nbc > 0) {
-    const int bcw = NS * 8 * 16;  // record of one inflow column: a group of 8, seven of them padding
-    for (int e = threadIdx.x; e < nbc * ar.oc * 8; e += blockDim.x) {
-      const int f = e / (ar.oc * 8), rem = e - f * ar.oc * 8, o = rem / 8, a = rem - o * 8;
+    // one inflow column: a group of 8, seven of them padding
+    const int co = ar.parts * ar.po;
+    for (int e = threadIdx.x; e < nbc * co * 8; e += blockDim.x) {
+      const int f = e / (co * 8), rem = e - f * co * 8, o = rem / 8, a = rem - o * 8;
       const int K = xg_shift_const(0.0, xg_unit(slots[ar.ncol + f], NS));
       unsigned dig[4][NS];
 #pragma unroll
@@ -362,11 +390,71 @@ __global__ void __launch_bounds__(256) k_xg_digits(const S* __restrict__ A, XgAr
         const double x1 = (a == 0 && g + 1 < ar.G) ? bc[f * ar.G + g + 1] : 0.0;
         xg_digits2<NS>(xg_fix(x0, K), xg_fix(x1, K), dig[u]);
       }
-      unsigned char* dst = bcout + (size_t)(f * ar.oc + o) * bcw;
 #pragma unroll
       for (int j = 0; j < NS; ++j)
-        *reinterpret_cast<uint4*>(dst + (j * 8 + a) * 16) = make_uint4(dig[0][j], dig[1][j], dig[2][j], dig[3][j]);
+        *reinterpret_cast<uint4*>(bcout + xg_dig_off<NS>((long)f * ar.parts + o / ar.po, ar.po, 8, j * 8 + a, o % ar.po)) =
+            make_uint4(dig[0][j], dig[1][j], dig[2][j], dig[3][j]);
     }
+  }
+}
+
+// Column maxima and digit records of a small explicit matrix in one launch: a CTA takes eight columns, all
+// rows (at most kXgSmallRows).  The small cores' matrices are a chain of short kernels, bound by
+// launches: this one stands for a memset and two kernels.  The first CTA zeroes the page of zeros.
+constexpr long kXgSmallRows = 4096;
+template <int NS, typename S>
+__global__ void __launch_bounds__(256) k_xg_small_digits(const S* __restrict__ A, XgArray ar, LivePattern lp, long nrows,
+                                                         unsigned long long* __restrict__ slots,
+                                                         unsigned char* __restrict__ out, uint4* __restrict__ zero,
+                                                         int nzero) {
+  constexpr int W = XgCfg<NS>::W;
+  __shared__ unsigned long long sm[8];
+  constexpr S kMax = sizeof(S) == 4 ? (S)3.402823466e+38f : (S)1.7976931348623157e308;
+  const int tid = threadIdx.x;
+  const int r = lp.r_ptr ? *lp.r_ptr : lp.rcap;
+  const int c0 = blockIdx.x * 8;
+  if (blockIdx.x == 0)
+    for (int i = tid; i < nzero; i += blockDim.x) zero[i] = make_uint4(0, 0, 0, 0);
+  if (tid < 8) sm[tid] = 0ull;
+  __syncthreads();
+  // maxima: the faster of rows and columns in memory goes along the lanes
+  const bool rowmajor = ar.sc == 1;
+  const int cl = rowmajor ? tid & 7 : tid >> 5, rl = rowmajor ? tid >> 3 : tid & 31;
+  {
+    const int c = c0 + cl;
+    S m = S(0);
+    if (c < ar.ncol && lp.live(c, r)) {
+#pragma unroll 8
+      for (long k = rl; k < nrows; k += 32) {
+        const S a = fabs(A[k * ar.sr + c * ar.sc]);
+        m = (a > m && a <= kMax) ? a : m;
+      }
+    }
+    atomicMax(&sm[cl], (unsigned long long)__double_as_longlong((double)m));
+  }
+  __syncthreads();
+  if (tid < 8 && c0 + tid < ar.ncol) slots[c0 + tid] = sm[tid];
+  const int cpad = ar.cpad;
+  const int noct = (int)ar.npiece * 8;  // cells of 64 rows: one piece of eight octets each
+  const int a8 = rowmajor ? tid & 7 : (tid >> 2) & 7;  // column of the slab
+  const int o0 = rowmajor ? tid >> 3 : (tid & 3) | ((tid >> 5) << 2);
+  const int c = c0 + a8;
+  const bool ok = c < ar.ncol && lp.live(c, r);
+  const int K = xg_shift_const(S(0), ok ? xg_unit(sm[a8], NS) : 0);
+  const int blk = c / W, a = c - blk * W;
+  const int w = cpad - blk * W < W ? cpad - blk * W : W;
+  for (int o = o0; o < noct; o += 32) {
+    S x[8];
+#pragma unroll
+    for (int u = 0; u < 8; ++u) x[u] = (ok && 8l * o + u < nrows) ? A[(8l * o + u) * ar.sr + c * ar.sc] : S(0);
+    unsigned dig[4][NS];
+#pragma unroll
+    for (int u = 0; u < 4; ++u) xg_digits2<NS>(xg_fix(x[2 * u], K), xg_fix(x[2 * u + 1], K), dig[u]);
+    unsigned char* dst = out + (size_t)(blk * W) * noct * (NS * 16);
+#pragma unroll
+    for (int j = 0; j < NS; ++j)
+      *reinterpret_cast<uint4*>(dst + xg_dig_off<NS>(o >> 3, 8, w, j * w + a, o & 7)) =
+          make_uint4(dig[0][j], dig[1][j], dig[2][j], dig[3][j]);
   }
 }
 
@@ -389,6 +477,11 @@ __device__ __forceinline__ void tmem_ld8(uint32_t taddr, uint32_t* r) {
                : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7])
                : "r"(taddr));
 }
+__device__ __forceinline__ void tmem_ld4(uint32_t taddr, uint32_t* r) {
+  asm volatile("tcgen05.ld.sync.aligned.32x32b.x4.b32 {%0, %1, %2, %3}, [%4];\n"
+               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
+               : "r"(taddr));
+}
 __device__ __forceinline__ void mbar_expect(uint64_t* bar, uint32_t bytes) {
   asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;\n" ::"r"(smem_u32(bar)), "r"(bytes) : "memory");
 }
@@ -403,61 +496,76 @@ __device__ __forceinline__ void bulk_g2s(uint32_t dst, const void* src, uint32_t
 }
 }  // namespace tc
 
-// Folds an accumulator tile into this thread's 64-bit sums: TMEM row m = this lane, columns of the right
-// block in groups of width WD: column n = (s NS + j) WD + b; acc[h][s WD + b] += 512^(..) value, digits
-// j < 4 into h = 0 and the rest into h = 1.
-template <int NS, int WD>
-__device__ __forceinline__ void xg_fold(uint32_t ta, int nsub, long long* acc) {
-  constexpr int W = XgCfg<NS>::W;
+// Columns of an operand block that one of the four folding warpgroups takes.
+template <int NS>
+struct XgFold {
+  static constexpr int Q = XgCfg<NS>::W / 4;
+};
+// Folds this warpgroup's columns of an accumulator tile into its 64-bit sums: TMEM row m = this lane, the
+// block's column c = s w + b at TMEM column (s NS + j) w + b for digit j (ta: at j = 0 of the first of Q
+// columns); acc[h][..] += 256^(..) value, digits j < 4 into h = 0 and the rest into h = 1.  All loads are in
+// flight at once; release (nullable): arrive there as soon as they have landed.
+template <int NS>
+__device__ __forceinline__ void xg_fold(uint32_t ta, int w, uint64_t* release, long long* acc) {
+  constexpr int Q = XgFold<NS>::Q;
+  uint32_t v[NS][Q];
 #pragma unroll
-  for (int s = 0; s < W / WD; ++s) {
-    if (s >= nsub) continue;
-#pragma unroll
-    for (int j = 0; j < NS; ++j) {
-      constexpr int CH = WD % 16 == 0 ? 16 : 8;  // columns in flight (registers hold the sums)
-      const int h = j / 4;
-      const int wgt = 1 << (9 * ((h == 0 ? 3 : NS - 1) - j));
-#pragma unroll
-      for (int b0 = 0; b0 < WD; b0 += CH) {
-        uint32_t v[CH];
-#pragma unroll
-        for (int b = 0; b < CH; b += 8) tc::tmem_ld8(ta + (uint32_t)((s * NS + j) * WD + b0 + b), v + b);
-        tc::tmem_wait_ld();
-#pragma unroll
-        for (int b = 0; b < CH; ++b)
-          asm("mad.wide.s32 %0, %1, %2, %0;"
-              : "+l"(acc[h * W + s * WD + b0 + b])
-              : "r"(__float2int_rn(__uint_as_float(v[b]))), "r"(wgt));
-      }
-    }
+  for (int j = 0; j < NS; ++j) {
+    if constexpr (Q == 8) tc::tmem_ld8(ta + (uint32_t)(j * w), v[j]);
+    else tc::tmem_ld4(ta + (uint32_t)(j * w), v[j]);
   }
+  tc::tmem_wait_ld();
+  if (release) {
+    tc::fence_before_sync();
+    __syncwarp();
+    if ((threadIdx.x & 31) == 0) tc::mbar_arrive(release);
+  }
+#pragma unroll
+  for (int j = 0; j < NS; ++j) {
+    const int wgt = 1 << (8 * (3 - j % 4));
+#pragma unroll
+    for (int b = 0; b < Q; ++b)
+      asm("mad.wide.s32 %0, %1, %2, %0;"
+          : "+l"(acc[(j / 4) * Q + b])
+          : "r"(__float2int_rn(__uint_as_float(v[j][b]))), "r"(wgt));
+  }
+}
+
+// Whether MMA group g ends a chunk with tile t (of ntile): the two groups' chunks are half a chunk apart.
+__device__ __forceinline__ bool xg_ends(int g, int t, int ntile) {
+  return (t + 1 + g * (kXgChunkTiles / 2)) % kXgChunkTiles == 0 || t == ntile - 1;
 }
 
 // The digit products of a row range: CTA (group, k) accumulates the tiles of plan entry k over its row
 // group and writes its 64-bit sums to part[group][tile][h][column n][row m].  One warp copies the
-// operand blocks of 64 rows into a ring of stages (one bulk copy per column group and octet), one
-// thread issues the MMAs, and four warps per tile fold its accumulators every 256 rows; the tiles' fold
-// points are staggered by 64 rows, so the MMAs of the other tiles run while one is folded.
+// operand blocks of up to 64 rows into a ring of stages (one bulk copy per column group and piece: copies
+// an octet at a time, 2 KB, took 1.6 times as long), one thread issues the MMAs, and sixteen warps fold a
+// group's accumulators every 16 stages (at most 1024 rows; each warp a quarter of the rows and of the
+// columns, all its loads in flight) while the MMAs of the other group run.  Bound by the MMAs.
 template <int NS>
 __global__ void __launch_bounds__(kXgThreads, 1)
     k_xg_mma(const __grid_constant__ XgPlan pl, const __grid_constant__ XgArgs ar, long long* __restrict__ part,
              int* __restrict__ status) {
-  constexpr int W = XgCfg<NS>::W, H = XgCfg<NS>::H, NSW = NS * W;
+  constexpr int W = XgCfg<NS>::W, H = XgCfg<NS>::H;
   extern __shared__ __align__(1024) unsigned char xg_smem[];
-  __shared__ uint64_t full[kXgMaxStage], empty[kXgMaxStage], acc_full[kXgTiles], acc_empty[kXgTiles];
-  __shared__ uint32_t tbase, boff[kXgMaxBlk];
+  __shared__ uint64_t full[kXgMaxStage], empty[kXgMaxStage], acc_full[kXgGroups], acc_empty[kXgGroups];
+  __shared__ uint32_t tbase, rows_s;
   __shared__ int nsubs;
   __shared__ struct {
-    uint32_t dst, ldo;  // smem offset of the group in its stage, bytes per octet of its block
-    int off, bytes, arr, nb;
+    uint64_t a, b;
+    uint32_t idesc;
+  } ginfo[kXgGroups];
+  __shared__ struct {
+    uint32_t dst;  // offset of the group in a piece of the stage
+    int c0, bytes, arr, nb;
   } csub[kXgMaxBlk * 4];
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int kcta = blockIdx.x % pl.ncta;
   const long group = blockIdx.x / pl.ncta;
-  const int nblk = pl.cblks[kcta], nt = pl.ctiles[kcta], nst = ar.nstage;
-  const uint32_t ncols = tc::tmem_cols(nt * NSW);
+  const int nblk = pl.cblks[kcta], ng = pl.cgroups[kcta], nst = ar.nstage;
+  constexpr uint32_t kCols = 512;
   if (warp == 0) {
-    tc::tmem_alloc(&tbase, ncols);
+    tc::tmem_alloc(&tbase, kCols);
     tc::tmem_relinquish();
   }
   if (tid == 32) {
@@ -465,30 +573,45 @@ __global__ void __launch_bounds__(kXgThreads, 1)
       tc::mbar_init(&full[i], 1);
       tc::mbar_init(&empty[i], 1);
     }
-    for (int i = 0; i < kXgTiles; ++i) {
+    for (int i = 0; i < kXgGroups; ++i) {
       tc::mbar_init(&acc_full[i], 1);
-      tc::mbar_init(&acc_empty[i], 4);
+      tc::mbar_init(&acc_empty[i], 16);
     }
-    uint32_t o = 0;
+    // a piece of a stage: the rows (digits of columns) of the CTA's blocks one after the other, in eights
+    // of po octets each (K-major core matrices without swizzle: LBO 128, SBO 128 po)
+    const uint32_t po16 = (uint32_t)ar.po * 16u;
+    uint32_t rows = 0, boff[kXgMaxBlk];
     int n = 0;
     for (int i = 0; i < nblk; ++i) {
-      const int b = pl.blk[kcta][i], rows = xg_block_rows(pl, b);
-      boff[i] = o;
+      const int b = pl.blk[kcta][i];
+      boff[i] = rows;
       for (int u = 0; u < pl.bnsub[b]; ++u) {
         const XgSub& sb = pl.sub[pl.bsub0[b] + u];
-        csub[n].dst = o + (uint32_t)(u * NS * sb.w) * 16u;
-        csub[n].ldo = (uint32_t)rows * 16u;
-        csub[n].off = sb.off;
-        csub[n].bytes = NS * sb.w * 16;
+        csub[n].dst = (rows + (uint32_t)(u * NS * sb.w)) * po16;
+        csub[n].c0 = sb.c0;
+        csub[n].bytes = NS * sb.w * (int)po16;
         csub[n].arr = sb.arr;
         csub[n].nb = sb.nb;
         ++n;
       }
-      o += (uint32_t)rows * 128u;
+      rows += (uint32_t)xg_block_rows(pl, b);
     }
     nsubs = n;
+    rows_s = rows;
+    // operands of the MMA groups: descriptors at stage 0 (the address field counts 16 bytes) and the
+    // instruction descriptor, read by the issuing thread for every stage (from the plan in constant
+    // memory the chain of dependent loads took longer than the MMAs)
+    const uint32_t s0 = tc::smem_u32(xg_smem);
+    for (int g = 0; g < ng; ++g) {
+      const int m = pl.gm[kcta][g], n0 = pl.gn[kcta][g];
+      int nrow = 0;
+      for (int i = 0; i < pl.gnn[kcta][g]; ++i) nrow += xg_block_rows(pl, pl.blk[kcta][n0 + i]);
+      ginfo[g].a = tc::smem_desc(s0 + boff[m] * po16, 128u, 8u * po16);
+      ginfo[g].b = tc::smem_desc(s0 + boff[n0] * po16, 128u, 8u * po16);
+      ginfo[g].idesc = tc::idesc_f16(128, nrow);
+    }
   }
-  // what an M = 128 operand may read past the last stage
+  // what an M = 128 operand may read past the last piece
   for (int i = tid; i < (int)kXgPad / 16; i += kXgThreads)
     reinterpret_cast<uint4*>(xg_smem + nst * ar.stage_bytes)[i] = make_uint4(0, 0, 0, 0);
   tc::fence_before_sync();
@@ -496,89 +619,100 @@ __global__ void __launch_bounds__(kXgThreads, 1)
   tc::fence_after_sync();
   const uint32_t tmem = tbase;
   const uint32_t sbase = tc::smem_u32(xg_smem);
-  const long ob = group * ar.opg;
-  const long oe = (ob + ar.opg < ar.noct) ? ob + ar.opg : ar.noct;
-  const int ntile = (int)((oe - ob + 7) / 8);
+  const uint32_t pieceb = rows_s * (uint32_t)ar.po * 16u;  // bytes of a piece of the stage
+  const int nc = ar.nc;
+  const long pb = group * ar.ppg;
+  const long pe = (pb + ar.ppg < ar.npiece) ? pb + ar.ppg : ar.npiece;
+  const int ntile = (int)((pe - pb + nc - 1) / nc);
   bool lost = false;  // a bounded wait of this thread ran out
 
   if (warp < 16) {
-    // ---- fold
-    const int q = warp >> 2;
-    if (q < nt) {
-      long long acc[W * H];
+    // ---- fold: warpgroup v takes the columns [v Q, v Q + Q) of every tile's right block
+    constexpr int Q = XgFold<NS>::Q;
+    const int v = warp >> 2;
+    long long acc[kXgTiles][H * Q];
+    uint32_t ta[kXgTiles];
+    int wd[kXgTiles];
 #pragma unroll
-      for (int i = 0; i < W * H; ++i) acc[i] = 0;
-      const int bq = pl.blk[kcta][pl.tq[kcta][q]];
-      const int w = pl.sub[pl.bsub0[bq]].w, ns = pl.bnsub[bq];
-      const uint32_t ta = tmem + ((uint32_t)(32 * (warp & 3)) << 16) + (uint32_t)(q * NSW);
-      int f = 0;
-      for (int t = 0; t < ntile && !lost; ++t) {
-        if (!((t + 1 - q) % 4 == 0 || t == ntile - 1)) continue;
-        if (!tc::mbar_wait(&acc_full[q], f & 1)) {
-          lost = true;
-          break;
-        }
-        ++f;
-        tc::fence_after_sync();
-        if constexpr (NS == 4) {
-          if (w == 32) xg_fold<NS, 32>(ta, ns, acc);
-          else if (w == 24) xg_fold<NS, 24>(ta, ns, acc);
-          else if (w == 16) xg_fold<NS, 16>(ta, ns, acc);
-          else xg_fold<NS, 8>(ta, ns, acc);
-        } else {
-          if (w == 16) xg_fold<NS, 16>(ta, ns, acc);
-          else xg_fold<NS, 8>(ta, ns, acc);
-        }
-        tc::fence_before_sync();
-        __syncwarp();
-        if (lane == 0) tc::mbar_arrive(&acc_empty[q]);
+    for (int q = 0; q < kXgTiles; ++q) {
+#pragma unroll
+      for (int i = 0; i < H * Q; ++i) acc[q][i] = 0;
+      wd[q] = 0;
+      ta[q] = 0;
+      if (pl.tp[kXgTiles * kcta + q] != 255) {
+        const int bq = pl.tq[kXgTiles * kcta + q];
+        const int w = pl.sub[pl.bsub0[bq]].w, sb = (v * Q) / w;
+        if (sb < pl.bnsub[bq]) wd[q] = w;  // 0: no such columns
+        const int first = (q & 1) ? xg_block_rows(pl, bq - 1) : 0;  // the pair's first block
+        ta[q] = tmem + ((uint32_t)(32 * (warp & 3)) << 16) + (uint32_t)((q >> 1) * 256 + first + sb * NS * w + (v * Q - sb * w));
       }
-      long long* out = part + ((size_t)group * pl.ntile + pl.tile0[kcta] + q) * (size_t)(H * W * 128);
-      const int m = 32 * (warp & 3) + lane;
+    }
+    int f[kXgGroups] = {0, 0};
+    for (int t = 0; t < ntile && !lost; ++t) {
 #pragma unroll
-      for (int i = 0; i < W * H; ++i) out[(size_t)i * 128 + m] = acc[i];
+      for (int g = 0; g < kXgGroups; ++g) {
+        if (g >= ng || lost || !xg_ends(g, t, ntile)) continue;
+        if (!tc::mbar_wait(&acc_full[g], f[g] & 1)) {
+          lost = true;
+          continue;
+        }
+        ++f[g];
+        tc::fence_after_sync();
+        if (wd[2 * g] > 0) xg_fold<NS>(ta[2 * g], wd[2 * g], wd[2 * g + 1] > 0 ? nullptr : &acc_empty[g], acc[2 * g]);
+        if (wd[2 * g + 1] > 0) xg_fold<NS>(ta[2 * g + 1], wd[2 * g + 1], &acc_empty[g], acc[2 * g + 1]);
+        if (wd[2 * g] == 0 && wd[2 * g + 1] == 0 && lane == 0) tc::mbar_arrive(&acc_empty[g]);
+      }
+    }
+    const int m = 32 * (warp & 3) + lane;
+#pragma unroll
+    for (int q = 0; q < kXgTiles; ++q) {
+      if (pl.tp[kXgTiles * kcta + q] == 255) continue;
+      long long* out = part + ((size_t)group * pl.ncta * kXgTiles + kXgTiles * kcta + q) * (size_t)(H * W * 128);
+#pragma unroll
+      for (int h = 0; h < H; ++h)
+#pragma unroll
+        for (int b = 0; b < Q; ++b) out[(size_t)(h * W + v * Q + b) * 128 + m] = acc[q][h * Q + b];
     }
   } else if (warp == 16) {
     // ---- copies
-    const int n8 = nsubs * 8;
-    uint32_t total = 0;
-    for (int i = 0; i < nsubs; ++i) total += (uint32_t)csub[i].bytes * 8u;
+    const int ncopy = nsubs * nc;
     for (int t = 0; t < ntile; ++t) {
       const int st = t % nst, ph = t / nst;
       if (t >= nst && !tc::mbar_wait(&empty[st], (ph - 1) & 1)) {
         lost = true;
         break;
       }
-      if (lane == 0) tc::mbar_expect(&full[st], total);
+      if (lane == 0) tc::mbar_expect(&full[st], pieceb * (uint32_t)nc);
       __syncwarp();
       const uint32_t stage = sbase + (uint32_t)(st * ar.stage_bytes);
-      for (int i = lane; i < n8; i += 32) {
-        const int u = i >> 3, o = i & 7;
-        const long oct = ob + (long)t * 8 + o;
-        const int nb = csub[u].nb;
+      for (int i = lane; i < ncopy; i += 32) {
+        const int u = i / nc, c = i - u * nc;
+        const long piece = pb + (long)t * nc + c;
+        const int nb = csub[u].nb, bytes = csub[u].bytes;
         const unsigned char* src = ar.zero;
-        if (oct < oe && nb != 255) {
-          long from = oct;
+        if (piece < pe) {
+          long from = piece;
           bool ok = true;
           if (nb != 0) {
-            const unsigned cell = (unsigned)oct / (unsigned)ar.oc;
+            const unsigned cell = (unsigned)piece / (unsigned)ar.parts;
             if (nb < 8) {
               const int ax = (nb - 1) >> 1, up = (nb - 1) & 1;
               const int idx = (int)((cell / (unsigned)ar.cstr[ax]) % (unsigned)ar.ext[ax]);
               ok = up ? idx < ar.ext[ax] - 1 : idx > 0;
-              from += (up ? 1L : -1L) * ar.cstr[ax] * ar.oc;
+              from += (up ? 1L : -1L) * ar.cstr[ax] * ar.parts;
             } else {
               const int face = ar.face[nb - 8], ax = face >> 1;
               const int idx = (int)((cell / (unsigned)ar.cstr[ax]) % (unsigned)ar.ext[ax]);
               ok = (face & 1) ? idx == ar.ext[ax] - 1 : idx == 0;
-              from = (long)(nb - 8) * ar.oc + (oct - (long)cell * ar.oc);
+              from = (long)(nb - 8) * ar.parts + (piece - (long)cell * ar.parts);
             }
           }
           if (ok)
-            src = nb >= 8 ? ar.bc + from * ar.bcrec
-                          : (csub[u].arr ? ar.dig[1] + from * ar.rec[1] : ar.dig[0] + from * ar.rec[0]) + csub[u].off;
+            src = nb >= 8 ? ar.bc + from * bytes
+                          : (csub[u].arr ? ar.dig[1] : ar.dig[0]) +
+                                (size_t)csub[u].c0 * ar.npiece * (ar.po * NS * 16) + from * bytes;
         }
-        tc::bulk_g2s(stage + csub[u].dst + (uint32_t)o * csub[u].ldo, src, (uint32_t)csub[u].bytes, &full[st]);
+        tc::bulk_g2s(stage + (uint32_t)c * pieceb + csub[u].dst, src, (uint32_t)bytes, &full[st]);
       }
     }
     // the copies in flight land before the CTA ends (their stages were all consumed otherwise)
@@ -587,7 +721,10 @@ __global__ void __launch_bounds__(kXgThreads, 1)
         if (st < ntile) (void)tc::mbar_wait(&full[st], 0, 1L << 16);
   } else if (lane == 0) {
     // ---- MMAs
-    int used[kXgTiles] = {0, 0, 0, 0};  // chunks folded so far
+    // K steps of two octets; pieces of 1, 2, 3 or 4 steps (3 and 4: one piece a stage)
+    const int pk = ar.po / 2, ksteps = nc * pk, psh = pk < 3 ? pk - 1 : 2;
+    int folds[kXgGroups] = {0, 0};        // chunks ended so far
+    bool fresh[kXgGroups] = {true, true}; // the next MMA of the group starts a chunk
     for (int t = 0; t < ntile; ++t) {
       const int st = t % nst;
       if (!tc::mbar_wait(&full[st], (t / nst) & 1)) {
@@ -595,31 +732,38 @@ __global__ void __launch_bounds__(kXgThreads, 1)
         break;
       }
       tc::fence_after_sync();
-      const uint32_t stage = sbase + (uint32_t)(st * ar.stage_bytes);
+      const uint32_t so = (uint32_t)(st * ar.stage_bytes) >> 4;
+      // a group whose accumulators are being folded comes last
+      const bool swap = fresh[0] && folds[0] > 0;
 #pragma unroll
-      for (int i = 0; i < kXgTiles; ++i) {
-        const int q = (t + 1 + i) & 3;  // the tile that starts a chunk here comes last
-        if (q >= nt) continue;
-        const bool start = t == 0 || (t - q) % 4 == 0;
-        if (start && t > 0 && !lost) {
-          int u = 0;
-#pragma unroll
-          for (int x = 0; x < kXgTiles; ++x)
-            if (x == q) u = used[x]++;
-          if (!tc::mbar_wait(&acc_empty[q], u & 1)) lost = true;
+      for (int i = 0; i < kXgGroups; ++i) {
+        const int g = swap ? 1 - i : i;
+        if (g >= ng || lost) continue;
+        const bool start = g == 0 ? fresh[0] : fresh[1];
+        const int done = g == 0 ? folds[0] : folds[1];
+        if (start && done > 0) {
+          if (!tc::mbar_wait(&acc_empty[g], (done - 1) & 1)) lost = true;
           tc::fence_after_sync();
+          if (lost) continue;
         }
-        if (lost) break;
-        const int lp = pl.tp[kcta][q], lq = pl.tq[kcta][q];
-        const int rp = xg_block_rows(pl, pl.blk[kcta][lp]), rq = xg_block_rows(pl, pl.blk[kcta][lq]);
-        const uint32_t ldp = (uint32_t)rp * 16u, ldq = (uint32_t)rq * 16u;
-        const uint32_t ap = stage + boff[lp], bp = stage + boff[lq];
-        const uint32_t idesc = tc::idesc_f16(128, rq);
+        const uint64_t da = ginfo[g].a + so, db = ginfo[g].b + so;
+        const uint32_t idesc = ginfo[g].idesc, d = tmem + (uint32_t)(g * 256);
 #pragma unroll
-        for (int kk = 0; kk < 4; ++kk)
-          tc::mma_f16(tmem + (uint32_t)(q * NSW), tc::smem_desc(ap + 2u * kk * ldp, ldp, 128u),
-                      tc::smem_desc(bp + 2u * kk * ldq, ldq, 128u), idesc, (start && kk == 0) ? 0u : 1u);
-        if ((t + 1 - q) % 4 == 0 || t == ntile - 1) tc::mma_commit(&acc_full[q]);
+        for (int kk = 0; kk < 4; ++kk) {
+          if (kk >= ksteps) break;
+          const int c = kk >> psh;
+          const uint32_t k = ((uint32_t)c * pieceb + (uint32_t)(kk - c * pk) * 256u) >> 4;
+          tc::mma_f16(d, da + k, db + k, idesc, (start && kk == 0) ? 0u : 1u);
+        }
+        const bool ends = xg_ends(g, t, ntile);
+        if (ends) tc::mma_commit(&acc_full[g]);
+        if (g == 0) {
+          fresh[0] = ends;
+          folds[0] += ends;
+        } else {
+          fresh[1] = ends;
+          folds[1] += ends;
+        }
       }
       if (lost) break;
       tc::mma_commit(&empty[st]);
@@ -634,7 +778,7 @@ __global__ void __launch_bounds__(kXgThreads, 1)
   if (__syncthreads_or(lost) && tid == 0) latch(status, TT_ERR_TIMEOUT);
   if (warp == 0) {
     tc::fence_after_sync();
-    tc::tmem_dealloc(tmem, ncols);
+    tc::tmem_dealloc(tmem, kCols);
   }
 }
 
@@ -668,13 +812,21 @@ __device__ __forceinline__ void add_shifted(Int192& a, __int128 v, int sh) {  //
 // Raw products as 192-bit integers, summed over the row groups, the left digits i and the digit groups of
 // the right column: gint[word plane][row a][column b], row-major with ldg.  Upper triangle of blocks: the
 // mirrored entry is written too; split: columns of array 1 start at ldg's column 0.  One thread per entry.
+// unit, coef (nullable): the columns' units and coefficients where the raw columns are the columns.
 template <int NS>
 __global__ void __launch_bounds__(256) k_xg_sum(const __grid_constant__ XgPlan pl, int ngroups, int split, int ldg,
                                                 size_t plane, const long long* __restrict__ part,
-                                                unsigned long long* __restrict__ gint) {
+                                                unsigned long long* __restrict__ gint,
+                                                const unsigned long long* __restrict__ slots, int* __restrict__ unit,
+                                                double* __restrict__ coef) {
   constexpr int W = XgCfg<NS>::W, H = XgCfg<NS>::H;
+  if (unit && blockIdx.x == 0 && blockIdx.y == 0 && (int)threadIdx.x < ldg) {
+    unit[threadIdx.x] = xg_unit(slots[threadIdx.x], NS);
+    coef[threadIdx.x] = 1.0;
+  }
   const int tile = blockIdx.x;
-  const int p = pl.gp[tile], q = pl.gq[tile];
+  const int p = pl.tp[tile], q = pl.tq[tile];
+  if (p == 255) return;
   const int idx = blockIdx.y * blockDim.x + threadIdx.x;
   const int ia = idx % W, ib = idx / W;
   if (ib >= W) return;
@@ -685,7 +837,7 @@ __global__ void __launch_bounds__(256) k_xg_sum(const __grid_constant__ XgPlan p
   const XgSub& uq = pl.sub[pl.bsub0[q] + sq];
   const int a = ia - sp * wp, b = ib - sq * wq;
   if (a >= up.cnt || b >= uq.cnt) return;
-  const size_t gstride = (size_t)pl.ntile * (H * W * 128);
+  const size_t gstride = (size_t)pl.ncta * kXgTiles * (H * W * 128);
   const long long* base = part + (size_t)tile * (H * W * 128);
   Int192 g{{0ull, 0ull, 0ull}};
 #pragma unroll
@@ -703,7 +855,7 @@ __global__ void __launch_bounds__(256) k_xg_sum(const __grid_constant__ XgPlan p
         for (int u = 0; u < 8; ++u) s += v[u];
       }
       for (; gr < ngroups; ++gr) s += ptr[gr * gstride];
-      add_shifted(g, s, 9 * (NS - 1 - i) + ((H == 2 && h == 0) ? 9 * (NS - 4) : 0));
+      add_shifted(g, s, 8 * (NS - 1 - i) + 8 * 4 * (H - 1 - h));
     }
   }
   const int ra = up.raw0 + a, rb = uq.raw0 + b - split;
@@ -749,11 +901,6 @@ __device__ __forceinline__ XgComb xg_comb(const SrcStencil<S>& s, int c) {
   else { put(Hh, 1); put(C, -1); }
   return x;
 }
-template <class Src>
-__device__ __forceinline__ XgComb xg_comb(const Src&, int c) {
-  return XgComb{1, {c, 0, 0}, {1, 0, 0}, c, 1.0};
-}
-
 // Upper triangle of the Gram matrix of the sum's columns from the raw products (exact), and each
 // column's unit and coefficient.
 template <int NS, class Src>
@@ -794,27 +941,27 @@ __global__ void __launch_bounds__(256) k_xg_combine(const __grid_constant__ Src 
 }
 
 // ---- host drivers --------------------------------------------------------------------------------
-// Row groups of a pass: one CTA per SM over ncta CTAs a group (`sms` SMs for this pass), at least 128
-// rows each, and at most kXgMaxOct octets.
-inline void xg_groups(long noct, int ncta, int sms, long& groups, long& opg) {
+// Row groups of a pass: one CTA per SM over ncta CTAs a group (`sms` SMs for this pass), at least two
+// stages each, and at most kXgMaxPieces.
+inline void xg_groups(long npiece, int nc, int ncta, int sms, long& groups, long& ppg) {
   groups = sms / ncta;
-  const long most = (noct + 15) / 16, least = (noct + kXgMaxOct - 1) / kXgMaxOct;
+  const long most = (npiece + 2 * nc - 1) / (2 * nc), least = (npiece + kXgMaxPieces - 1) / kXgMaxPieces;
   if (groups > most) groups = most;
   if (groups < least) groups = least;
   if (groups < 1) groups = 1;
-  opg = (noct + groups - 1) / groups;
-  opg = (opg + 7) / 8 * 8;
-  groups = (noct + opg - 1) / opg;
+  ppg = (npiece + groups - 1) / groups;
+  ppg = (ppg + nc - 1) / nc * nc;
+  groups = (npiece + ppg - 1) / ppg;
 }
 
 template <class Src>
 struct XgElem;
 template <typename S>
-struct XgElem<SrcRows<S>> { using type = S; };
+struct XgElem<SrcRows<S>> { using type = S; static constexpr bool stencil = false; };
 template <typename S>
-struct XgElem<SrcCols<S>> { using type = S; };
+struct XgElem<SrcCols<S>> { using type = S; static constexpr bool stencil = false; };
 template <typename S>
-struct XgElem<SrcStencil<S>> { using type = S; };
+struct XgElem<SrcStencil<S>> { using type = S; static constexpr bool stencil = true; };
 
 // Plan of a source's columns.
 template <int NS, typename S>
@@ -840,24 +987,27 @@ inline bool xg_make_plan(const SrcStencil<S>& s, const LivePattern& lp, XgPlan& 
     if (!xg_add<NS>(pl, 1, nsh * s.rcap + e, 0, 8 + e)) return false;
   return xg_tiles<NS>(pl, false) && xg_stages(pl) >= 2;
 }
+inline int xg_cpad(int n) { return (n + 7) & ~7; }
 template <typename S>
-inline bool xg_array(const SrcRows<S>& s, int n, long nrows, int NS, XgArray& ar, const S** A) {
-  ar = XgArray{n, 8, 1, (nrows + 7) / 8, NS == 4 ? xg_record<4>(n) : xg_record<7>(n), s.ld, 1};
+inline bool xg_array(const SrcRows<S>& s, int n, long nrows, XgArray& ar, const S** A) {
+  ar = XgArray{n, 64, 0, 0, (nrows + 63) / 64, 0, xg_cpad(n), s.ld, 1};
+  xg_pieces(ar);
   *A = s.A;
-  return ar.ncell < (1L << 31);
+  return ar.npiece < (1L << 28);
 }
 template <typename S>
-inline bool xg_array(const SrcCols<S>& s, int n, long nrows, int NS, XgArray& ar, const S** A) {
-  ar = XgArray{n, 8, 1, (nrows + 7) / 8, NS == 4 ? xg_record<4>(n) : xg_record<7>(n), 1, s.ld};
+inline bool xg_array(const SrcCols<S>& s, int n, long nrows, XgArray& ar, const S** A) {
+  ar = XgArray{n, 64, 0, 0, (nrows + 63) / 64, 0, xg_cpad(n), 1, s.ld};
+  xg_pieces(ar);
   *A = s.A;
-  return ar.ncell < (1L << 31);
+  return ar.npiece < (1L << 28);
 }
 template <typename S>
-inline bool xg_array(const SrcStencil<S>& s, int, long nrows, int NS, XgArray& ar, const S** A) {
-  ar = XgArray{s.rcap, s.G, (s.G + 7) / 8, nrows / s.G, NS == 4 ? xg_record<4>(s.rcap) : xg_record<7>(s.rcap),
-               s.ldz, 1};
+inline bool xg_array(const SrcStencil<S>& s, int, long nrows, XgArray& ar, const S** A) {
+  ar = XgArray{s.rcap, s.G, 0, 0, nrows / s.G, 0, xg_cpad(s.rcap), s.ldz, 1};
+  xg_pieces(ar);
   *A = s.Z;
-  return ar.ncell * ar.oc < (1L << 31);
+  return ar.npiece < (1L << 28);
 }
 template <class Src>
 inline LivePattern xg_array_live(const Src&, const LivePattern& lp) { return lp; }
@@ -910,16 +1060,17 @@ inline const XgPlan* xg_plan_of(const Src& src, const LivePattern& lp) {
 // Whether a pass of the source over nrows rows can take the exact Gram kernels.
 template <typename T, class Src>
 inline bool xg_fits(const Src& src, const LivePattern& lp, long nrows) {
-  constexpr int NS = sizeof(T) == 4 ? 4 : 7;
-  XgArray ar;
+  constexpr int NS = sizeof(T) == 4 ? 4 : 8;
+  XgArray ar{};
   const typename XgElem<Src>::type* A = nullptr;
-  return xg_plan_of<NS>(src, lp) != nullptr && xg_array(src, lp.ncap(), nrows, NS, ar, &A);
+  return xg_plan_of<NS>(src, lp) != nullptr && xg_array(src, lp.ncap(), nrows, ar, &A);
 }
 
 // Launches the product kernels of a plan whose digit records are in place.
 template <int NS>
 tt_status xg_launch_products(cudaStream_t s, const XgPlan& pl, XgArgs& args, long groups, long long* part, int split,
-                             int ldg, size_t plane, unsigned long long* gint, int* status) {
+                             int ldg, size_t plane, unsigned long long* gint, const unsigned long long* slots, int* unit,
+                             double* coef, int* status) {
   constexpr int W = XgCfg<NS>::W;
   args.stage_bytes = xg_stage_bytes(pl);
   args.nstage = xg_stages(pl);
@@ -929,8 +1080,8 @@ tt_status xg_launch_products(cudaStream_t s, const XgPlan& pl, XgArgs& args, lon
   if (const tt_status a = smem_optin(kern, smem); a != TT_OK) return a;
   kern<<<(unsigned)(groups * pl.ncta), kXgThreads, smem, s>>>(pl, args, part, status);
   count_launch();
-  k_xg_sum<NS><<<dim3((unsigned)pl.ntile, (W * W + 255) / 256), 256, 0, s>>>(pl, (int)groups, split, ldg, plane, part,
-                                                                           gint);
+  k_xg_sum<NS><<<dim3((unsigned)(pl.ncta * kXgTiles), (W * W + 255) / 256), 256, 0, s>>>(pl, (int)groups, split, ldg, plane, part,
+                                                                           gint, slots, unit, coef);
   count_launch();
   return cudaGetLastError() == cudaSuccess ? TT_OK : TT_ERR_CUDA;
 }
@@ -941,7 +1092,7 @@ void xg_launch_digits(cudaStream_t s, int num_sms, const S* A, const XgArray& ar
   long grid = need < 8L * num_sms ? need : 8L * num_sms;
   k_xg_colmax<S><<<(unsigned)(grid > 0 ? grid : 1), 256, 0, s>>>(A, ar.ncol, ar.sr, ar.sc, nrows, slots, bc, nbc, ar.G);
   count_launch();
-  const long tot = ar.ncell * ar.oc * (ar.rec / (NS * 16));
+  const long tot = ar.npiece * ar.po * ar.cpad;
   grid = (tot + 255) / 256;
   if (grid > 16L * num_sms) grid = 16L * num_sms;
   k_xg_digits<NS, S><<<(unsigned)(grid > 0 ? grid : 1), 256, 0, s>>>(A, ar, lp, nrows, slots, dig, bc, nbc, bcdig);
@@ -955,13 +1106,13 @@ template <typename T, class Src>
 tt_status xg_factor(cudaStream_t s, int num_sms, int sms, const Src& src, LivePattern lp, long nrows, Bump& ws,
                     double** RZ_out, int* status, int leaf_cat = kTsqrLeaf) {
   using S = typename XgElem<Src>::type;
-  constexpr int NS = sizeof(T) == 4 ? 4 : 7;
+  constexpr int NS = sizeof(T) == 4 ? 4 : 8;
   constexpr int W = XgCfg<NS>::W, H = XgCfg<NS>::H;
   const int n = lp.ncap();
   const XgPlan* plan = xg_plan_of<NS>(src, lp);
   XgArray ar;
   const S* A = nullptr;
-  if (!plan || !xg_array(src, n, nrows, NS, ar, &A)) return TT_ERR_UNSUPPORTED;
+  if (!plan || !xg_array(src, n, nrows, ar, &A)) return TT_ERR_UNSUPPORTED;
   const XgPlan& pl = *plan;
   double* R = ws.take<double>((size_t)n * n);
   *RZ_out = R;
@@ -971,40 +1122,50 @@ tt_status xg_factor(cudaStream_t s, int num_sms, int sms, const Src& src, LivePa
   const double* bc = nullptr;
   xg_geometry(src, args, &bc, &nbc);
   if (!bc) nbc = 0;
-  args.oc = ar.oc;
-  args.noct = ar.ncell * ar.oc;
-  args.rec[0] = ar.rec;
-  args.bcrec = NS * 8 * 16;
+  args.po = ar.po;
+  args.parts = ar.parts;
+  args.nc = 8 / ar.po;
+  args.npiece = ar.npiece;
   long groups;
-  xg_groups(args.noct, pl.ncta, sms > 0 ? sms : num_sms, groups, args.opg);
-  const size_t zbytes = (size_t)NS * W * 16;
+  xg_groups(args.npiece, args.nc, pl.ncta, sms > 0 ? sms : num_sms, groups, args.ppg);
+  constexpr bool direct = !XgElem<Src>::stencil;  // the raw columns are the columns
+  const bool small = direct && nrows <= kXgSmallRows;
+  const size_t zbytes = (size_t)8 * NS * W * 16;  // the largest piece of a column group
   // zeroed: column maxima and the page of zeros
   unsigned char* zeroed = ws.take<unsigned char>(zbytes + 8 * (size_t)(n + kMaxTerms));
   unsigned long long* slots = reinterpret_cast<unsigned long long*>(zeroed + zbytes);
-  unsigned char* dig = ws.take<unsigned char>((size_t)args.noct * ar.rec);
-  unsigned char* bcdig = ws.take<unsigned char>((size_t)nbc * ar.oc * args.bcrec);
-  long long* part = ws.take<long long>((size_t)groups * pl.ntile * (H * W * 128));
-  unsigned long long* raw = ws.take<unsigned long long>(3 * (size_t)pl.nraw * pl.nraw);
+  unsigned char* dig = ws.take<unsigned char>((size_t)ar.npiece * ar.po * ar.cpad * (NS * 16));
+  unsigned char* bcdig = ws.take<unsigned char>((size_t)nbc * ar.parts * ar.po * (NS * 8 * 16));
+  long long* part = ws.take<long long>((size_t)groups * pl.ncta * kXgTiles * (H * W * 128));
   unsigned long long* gint = ws.take<unsigned long long>(3 * (size_t)n * n);
+  unsigned long long* raw = direct ? gint : ws.take<unsigned long long>(3 * (size_t)pl.nraw * pl.nraw);
   int* unit = ws.take<int>(n);
   double* coef = ws.take<double>(n);
   ws.release(mark);
   if (ws.dry) return TT_OK;
   {
     TimerScope scope(leaf_cat, s);
-    cudaMemsetAsync(zeroed, 0, zbytes + 8 * (size_t)(n + kMaxTerms), s);
-    xg_launch_digits<NS>(s, num_sms, A, ar, xg_array_live(src, lp), nrows, slots, dig, bc, nbc, bcdig);
+    if (small) {
+      k_xg_small_digits<NS, S><<<(unsigned)((n + 7) / 8), 256, 0, s>>>(A, ar, lp, nrows, slots, dig,
+                                                                       reinterpret_cast<uint4*>(zeroed), (int)(zbytes / 16));
+      count_launch();
+    } else {
+      cudaMemsetAsync(zeroed, 0, zbytes + 8 * (size_t)(n + kMaxTerms), s);
+      xg_launch_digits<NS>(s, num_sms, A, ar, xg_array_live(src, lp), nrows, slots, dig, bc, nbc, bcdig);
+    }
     args.dig[0] = args.dig[1] = dig;
-    args.rec[1] = ar.rec;
     args.bc = bcdig;
     args.zero = zeroed;
-    const tt_status st = xg_launch_products<NS>(s, pl, args, groups, part, 0, pl.nraw,
-                                                (size_t)pl.nraw * pl.nraw, raw, status);
+    const tt_status st =
+        xg_launch_products<NS>(s, pl, args, groups, part, 0, pl.nraw, (size_t)pl.nraw * pl.nraw, raw, slots,
+                               direct ? unit : nullptr, direct ? coef : nullptr, status);
     if (st != TT_OK) return st;
-    k_xg_combine<NS, Src><<<(unsigned)((n * n + 255) / 256), 256, 0, s>>>(src, n, pl.nraw, raw, slots, gint, unit, coef);
-    count_launch();
+    if constexpr (!direct) {
+      k_xg_combine<NS, Src><<<(unsigned)((n * n + 255) / 256), 256, 0, s>>>(src, n, pl.nraw, raw, slots, gint, unit, coef);
+      count_launch();
+    }
   }
   TimerScope scope(kTsqrMerge, s);
-  return launch_xg_chol(s, n, gint, unit, coef, R);
+  return launch_xg_chol<(NS == 4 ? 1 : 2)>(s, n, gint, unit, coef, R);
 }
 }  // namespace ttk
