@@ -11,6 +11,7 @@
 #include "small.cuh"
 #include "step.cuh"
 #include "tc_update.cuh"
+#include "update_dig.cuh"
 #include "tsqr_blk.cuh"
 #include "tsqr_rs.cuh"
 #include "tune.cuh"
@@ -221,8 +222,9 @@ static tt_status launch_update_blk(cudaStream_t s, int num_sms, const SrcStencil
 template <typename T, class Src, class Epi>
 static tt_status launch_update(const tt_context* ctx, cudaStream_t s, int num_sms, const Src& src, LivePattern lp,
                                long nrows, const double* W, int kcap, const Epi& epi, double* partials,
-                               long* grid_out, int cat = kUpdate) {
+                               long* grid_out, int cat = kUpdate, const UdBufs* ub = nullptr) {
   constexpr int TM = UpdTM<T>::value;
+  if (ub && ub->rinfo) return launch_update_dig<T>(s, num_sms, src, lp, *ub, nrows, W, kcap, epi, partials, grid_out, cat);
   if constexpr (sizeof(T) == 4 && std::is_same<Src, SrcStencil<float>>::value) {
     if (ctx->tensor_cores && update_tc_fits(src, lp, nrows, kcap, ctx->smem_optin))
       return launch_update_tc(s, num_sms, src, lp, nrows, W, kcap, epi, partials, grid_out, cat);
@@ -303,6 +305,22 @@ inline int xg_sms(const tt_context* ctx) {
   if (ctx->tsqr_leaf_cap <= 0) return ctx->num_sms;
   const int share = (ctx->tsqr_leaf_cap + BigLeaves<T>::per_sm - 1) / BigLeaves<T>::per_sm;
   return share < ctx->num_sms ? share : ctx->num_sms;
+}
+
+// Whether a pass's update runs from digits on the tensor cores (update_dig.cuh), and its buffers.
+template <typename T, class Src>
+inline bool take_ud(const tt_context* ctx, const Src& src, const LivePattern& lp, long nrows, int kcap, Bump& ws,
+                    UdBufs& ub) {
+  if (ctx->no_xg || !update_dig_fits<T>(src, lp, nrows, kcap)) return false;
+  if constexpr (sizeof(T) == 4 && std::is_same<Src, SrcStencil<float>>::value) {
+    if (ctx->tensor_cores && nrows < kUdMinRowsTc && update_tc_fits(src, lp, nrows, kcap, ctx->smem_optin)) return false;
+  }
+  ub.cexp = ws.take<int>(lp.ncap());
+  if (XgElem<Src>::stencil) ub.rho = ws.take<short>(nrows);
+  ub.w = ws.take<unsigned char>(update_dig_wbytes<T>(src, lp, kcap));
+  int* rinfo = ws.take<int>(nrows);
+  ub.rinfo = ws.dry ? nullptr : rinfo;
+  return !ws.dry;
 }
 
 // Workspace carving shared by dry runs (size queries) and real runs.
@@ -452,10 +470,13 @@ tt_status round_impl(tt_context* ctx, tt_tensor* x, double tol, int rmax, Bump& 
     if (st != TT_OK) return st;
   }
   job.RZ = RZ;
-  tt_status st = small_round(s, ctx->num_sms, job, ws);
+  UdBufs ub;
+  tt_status st = TT_OK;
+  if (take_ud<T>(ctx, src, lp, N, K1, ws, ub)) st = launch_ud_scales(s, RZ, R, ub);
+  if (st == TT_OK) st = small_round(s, ctx->num_sms, job, ws);
   if (st != TT_OK || ws.dry) return st;
   st = launch_update<T>(ctx, s, ctx->num_sms, SrcRows<S>{(const S*)x->core[0], K1}, lp, N, b.W, K1,
-                        EpiPlain<S>{(S*)x->core[0], K1, &ctx->ctrl->status}, nullptr, nullptr);
+                        EpiPlain<S>{(S*)x->core[0], K1, &ctx->ctrl->status}, nullptr, nullptr, kUpdate, &ub);
   if (st != TT_OK) return st;
   const long tot = (long)K1 * n1 * K2 + (long)K2 * n2;
   k_commit<S><<<(unsigned)((tot + 255) / 256), 256, 0, s>>>(d, n1, n2, K1, K2, b.core1, b.core2,
@@ -541,7 +562,10 @@ tt_status step_impl(tt_context* ctx, const tt_plan* p, tt_tensor* I, double tol,
     if (st != TT_OK) return st;
   }
   j1.RZ = RZ1;
-  tt_status st = small_round(s, ctx->num_sms, j1, ws);
+  UdBufs ub1, ub2;
+  tt_status st = TT_OK;
+  if (take_ud<T>(ctx, src1, lp1, N, K1, ws, ub1)) st = launch_ud_scales(s, RZ1, R1, ub1);
+  if (st == TT_OK) st = small_round(s, ctx->num_sms, j1, ws);
   if (st != TT_OK) return st;
   // ---- source step fused into the write of the rounded transport update
   LivePattern lp2{nullptr, K1, 1, 1};
@@ -557,6 +581,7 @@ tt_status step_impl(tt_context* ctx, const tt_plan* p, tt_tensor* I, double tol,
   if (ws.dry) {
     SmallJob j2 = j1;
     j2.lp = lp2;
+    (void)take_ud<T>(ctx, SrcRows<S>{Zsrc, K1 + 1}, lp2, N, K1, ws, ub2);
     if (gram) {
       double* RZ2 = nullptr;
       st = gram_factor(s, ctx->num_sms, SrcRows<S>{Zsrc, K1 + 1}, lp2, N, ws, ctx->ctrl, ctx->coop_grid_max, &RZ2);
@@ -584,10 +609,11 @@ tt_status step_impl(tt_context* ctx, const tt_plan* p, tt_tensor* I, double tol,
   }
   st = launch_update<T>(ctx, s, ctx->num_sms, src1, lp1, N, b1.W, K1,
                         EpiSource<S>{Zsrc, K1 + 1, b1.vJ, p->acoef, p->scoef, p->eps, &ctx->ctrl->status}, part1,
-                        &ngrid1);
+                        &ngrid1, kUpdate, &ub1);
   if (st != TT_OK) return st;
   k_save_ranks<<<1, 32, 0, s>>>(ctx->ctrl); count_launch();
   lp2.r_ptr = &ctx->ctrl->k[2];
+  const bool ud2 = take_ud<T>(ctx, SrcRows<S>{Zsrc, K1 + 1}, lp2, N, K1, ws, ub2);
   // ---- second rounding: [D^-1 Z_new, g]
   k_b0_source<<<64, 256, 0, s>>>(K1, nang, b1.Bnew, b2.B0); count_launch();
   double* RZ2 = nullptr;
@@ -615,11 +641,12 @@ tt_status step_impl(tt_context* ctx, const tt_plan* p, tt_tensor* I, double tol,
   j2.core2 = b2.core2;
   j2.Bnew = b2.Bnew;
   j2.vJ = b2.vJ;
-  st = small_round(s, ctx->num_sms, j2, ws);
+  if (ud2) st = launch_ud_scales(s, RZ2, lp2.ncap(), ub2);
+  if (st == TT_OK) st = small_round(s, ctx->num_sms, j2, ws);
   if (st != TT_OK) return st;
   st = launch_update<T>(ctx, s, ctx->num_sms, SrcRows<S>{Zsrc, K1 + 1}, lp2, N, b2.W, K1,
                         EpiFinal<S>{(S*)I->core[0], K1, b2.vJ, jnew, &ctx->ctrl->status}, part2, &ngrid2,
-                        kUpdateSrc);
+                        kUpdateSrc, &ub2);
   if (st != TT_OK) return st;
   if (p->coupled) {
     st = coupled_t_update(s, const_cast<tt_plan*>(p), jstar, jnew);
