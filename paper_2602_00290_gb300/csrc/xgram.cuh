@@ -24,8 +24,8 @@
 // columns are written once (k_xg_digits, bound by memory) in the layout of the MMA operands, so that the
 // product kernel (k_xg_mma) only moves 16-byte rows with bulk copies: a neighbour block is the same
 // digits at another cell, a missing neighbour a page of zeros.  Measured for both roundings of a step
-// at 1,048,576 rows, rank 32: FP32 digits 0.18, products 0.67 ms (leaves and merges before: 6.0 + 2.1 ms);
-// FP64 0.28, 1.8 ms (before 99.6 + 14 ms).  With base 512 and MMAs of N = 128 columns over octets copied one by
+// at 1,048,576 rows, rank 32: FP32 digits 0.18, products 0.64 ms (leaves and merges before: 6.0 + 2.1 ms);
+// FP64 0.28, 1.7 ms (before 99.6 + 14 ms).  With base 512 and MMAs of N = 128 columns over octets copied one by
 // one the products took 0.87 and 3.06 ms.
 #pragma once
 #include <map>
@@ -39,15 +39,19 @@
 
 namespace ttk {
 
-constexpr int kXgThreads = 576;   // 16 folding warps, a copying warp, an MMA warp
+constexpr int kXgCopy = 2;        // copying warps
+constexpr int kXgThreads = 32 * (16 + kXgCopy + 1);  // 16 folding warps, the copying warps, an MMA warp
 constexpr int kXgGroups = 2;      // MMA groups of a CTA: one block of rows x up to two blocks (N <= 256)
 constexpr int kXgTiles = 4;       // output tiles of a CTA (TMEM: 4 x 128 columns)
-constexpr int kXgChunkTiles = 16; // tiles of 64 rows between two folds: 1024 * 2^14 = 2^24 is exact
+// Octets of rows of a stage (and at most of a piece): 64 rows.  A stage costs its hand-over beside its MMAs: with 32
+// rows the products of the 1,048,576 x 160 pass took 1.03 ms instead of 0.68 (FP64 2.80, 1.80).
+constexpr int kXgStageOct = 8;
+constexpr int kXgChunkTiles = 128 / kXgStageOct;  // stages between two folds: 1024 rows * 2^14 = 2^24 is exact
 constexpr int kXgMaxBlk = 6;      // operand blocks a CTA stages
 constexpr int kXgMaxSub = 56;     // column groups of a pass
 constexpr int kXgMaxNb = 24;      // operand blocks of a pass
 constexpr int kXgMaxCta = 80;     // CTAs that share a row range
-constexpr int kXgMaxStage = 6;
+constexpr int kXgMaxStage = 8;
 constexpr long kXgMaxPieces = 512L * 16;  // pieces per CTA: at most 512 chunks, the 64-bit sums stay below 2^58
 constexpr int kXgMaxRaw = 448;          // storage columns of all neighbour blocks
 
@@ -59,7 +63,7 @@ struct XgCfg {
 
 // A storage matrix whose rows are the groups of cells (row = g + G cell), or plain rows (cells of 64).  Its
 // digits are kept in pieces: a cell's rows (padded) in `parts` pieces of `po` octets, po even and at most
-// 8, so that a piece is a run of K for the MMAs and every neighbour's rows are pieces too.  One plane per
+// kXgStageOct, so that a piece is a run of K for the MMAs and every neighbour's rows are pieces too.  One plane per
 // column group: [cell][part][rows j w + a of the operand in eights][octet][8 rows x 16 bytes].
 struct XgArray {
   int ncol, G, po, parts;
@@ -69,7 +73,7 @@ struct XgArray {
 };
 inline void xg_pieces(XgArray& ar) {
   const int oc = (ar.G + 7) / 8;
-  ar.parts = (oc + 7) / 8;
+  ar.parts = (oc + kXgStageOct - 1) / kXgStageOct;
   ar.po = ((oc + ar.parts - 1) / ar.parts + 1) & ~1;
   ar.npiece = ar.ncell * ar.parts;
 }
@@ -231,19 +235,19 @@ inline bool xg_tiles(XgPlan& pl, bool split) {
   return true;
 }
 
-// Bytes of a stage (64 rows of every operand block of the CTA that stages most).
-inline size_t xg_stage_bytes(const XgPlan& pl) {
+// Bytes of a stage (every operand block of the CTA that stages most).
+inline size_t xg_stage_bytes(const XgPlan& pl, int oct = kXgStageOct) {
   size_t most = 0;
   for (int k = 0; k < pl.ncta; ++k) {
     size_t b = 0;
-    for (int i = 0; i < pl.cblks[k]; ++i) b += (size_t)xg_block_rows(pl, pl.blk[k][i]) * 128;
+    for (int i = 0; i < pl.cblks[k]; ++i) b += (size_t)xg_block_rows(pl, pl.blk[k][i]) * (16 * oct);
     if (b > most) most = b;
   }
   return most;
 }
 constexpr size_t kXgPad = 16 * 1024;  // an M = 128 operand of a narrower block reads past its piece
-inline int xg_stages(const XgPlan& pl) {
-  const int n = (int)((226 * 1024 - kXgPad) / xg_stage_bytes(pl));
+inline int xg_stages(const XgPlan& pl, int oct = kXgStageOct) {
+  const int n = (int)((226 * 1024 - kXgPad) / xg_stage_bytes(pl, oct));
   return n < kXgMaxStage ? n : kXgMaxStage;
 }
 
@@ -435,7 +439,7 @@ __global__ void __launch_bounds__(256) k_xg_small_digits(const S* __restrict__ A
   __syncthreads();
   if (tid < 8 && c0 + tid < ar.ncol) slots[c0 + tid] = sm[tid];
   const int cpad = ar.cpad;
-  const int noct = (int)ar.npiece * 8;  // cells of 64 rows: one piece of eight octets each
+  const int noct = (int)ar.npiece * ar.po;  // octets of rows, pieces one after the other
   const int a8 = rowmajor ? tid & 7 : (tid >> 2) & 7;  // column of the slab
   const int o0 = rowmajor ? tid >> 3 : (tid & 3) | ((tid >> 5) << 2);
   const int c = c0 + a8;
@@ -453,7 +457,7 @@ __global__ void __launch_bounds__(256) k_xg_small_digits(const S* __restrict__ A
     unsigned char* dst = out + (size_t)(blk * W) * noct * (NS * 16);
 #pragma unroll
     for (int j = 0; j < NS; ++j)
-      *reinterpret_cast<uint4*>(dst + xg_dig_off<NS>(o >> 3, 8, w, j * w + a, o & 7)) =
+      *reinterpret_cast<uint4*>(dst + xg_dig_off<NS>(o / ar.po, ar.po, w, j * w + a, o % ar.po)) =
           make_uint4(dig[0][j], dig[1][j], dig[2][j], dig[3][j]);
   }
 }
@@ -537,11 +541,12 @@ __device__ __forceinline__ bool xg_ends(int g, int t, int ntile) {
 }
 
 // The digit products of a row range: CTA (group, k) accumulates the tiles of plan entry k over its row
-// group and writes its 64-bit sums to part[group][tile][h][column n][row m].  One warp copies the
+// group and writes its 64-bit sums to part[group][tile][h][column n][row m].  Two warps copy the
 // operand blocks of up to 64 rows into a ring of stages (one bulk copy per column group and piece: copies
 // an octet at a time, 2 KB, took 1.6 times as long), one thread issues the MMAs, and sixteen warps fold a
 // group's accumulators every 16 stages (at most 1024 rows; each warp a quarter of the rows and of the
-// columns, all its loads in flight) while the MMAs of the other group run.  Bound by the MMAs.
+// columns, all its loads in flight) while the MMAs of the other group run.  A stage of eight MMAs (1,024 cycles at
+// the tensor cores' rate) takes about 1,800: the copies share the L2 (7 to 8 TB/s) and each stage is handed over.
 template <int NS>
 __global__ void __launch_bounds__(kXgThreads, 1)
     k_xg_mma(const __grid_constant__ XgPlan pl, const __grid_constant__ XgArgs ar, long long* __restrict__ part,
@@ -673,46 +678,70 @@ __global__ void __launch_bounds__(kXgThreads, 1)
 #pragma unroll
         for (int b = 0; b < Q; ++b) out[(size_t)(h * W + v * Q + b) * 128 + m] = acc[q][h * Q + b];
     }
-  } else if (warp == 16) {
-    // ---- copies
+  } else if (warp < 16 + kXgCopy) {
+    // ---- copies: a lane keeps some of a stage's copies, their sources and cells advanced from stage to
+    // stage (formed anew each time, with divisions and indexed parameters, the addresses of a stage took
+    // some 3,000 cycles: 8.3 ms of products at 3,538,944 x 242, then 6.6)
     const int ncopy = nsubs * nc;
+    constexpr int kPer = (kXgMaxBlk * 4 * (kXgStageOct / 2) + 32 * kXgCopy - 1) / (32 * kXgCopy);
+    const int first = lane * kXgCopy + (warp - 16);
+    const unsigned char* src[kPer];
+    uint32_t dst[kPer];
+    int bytes[kPer], kind[kPer], cs[kPer], ex[kPer], cpart[kPer], low[kPer], idx[kPer];
+    long piece[kPer];
+#pragma unroll
+    for (int k = 0; k < kPer; ++k) {
+      const int i = first + 32 * kXgCopy * k, u = i < ncopy ? i / nc : 0, c = i < ncopy ? i - u * nc : 0;
+      const int nb = csub[u].nb;
+      const int ax = nb == 0 ? 0 : nb < 8 ? (nb - 1) >> 1 : ar.face[nb - 8] >> 1;
+      bytes[k] = csub[u].bytes;
+      dst[k] = (uint32_t)c * pieceb + csub[u].dst;
+      // 0 the cell, 1 lower and 2 upper neighbour, 3 lower and 4 upper face
+      kind[k] = nb == 0 ? 0 : nb < 8 ? 1 + ((nb - 1) & 1) : 3 + (ar.face[nb - 8] & 1);
+      cs[k] = nb == 0 ? 1 : ar.cstr[ax];
+      ex[k] = nb == 0 ? 1 : ar.ext[ax];
+      piece[k] = i < ncopy ? pb + c : pe;
+      const long cell = piece[k] / ar.parts;
+      cpart[k] = (int)(piece[k] - cell * ar.parts);
+      low[k] = (int)(cell % cs[k]);
+      idx[k] = (int)((cell / cs[k]) % ex[k]);
+      const long shift = kind[k] == 1 ? -(long)cs[k] * ar.parts : kind[k] == 2 ? (long)cs[k] * ar.parts : 0;
+      src[k] = nb >= 8 ? ar.bc + (size_t)(nb - 8) * ar.parts * bytes[k]
+                       : (csub[u].arr ? ar.dig[1] : ar.dig[0]) + (size_t)csub[u].c0 * ar.npiece * (ar.po * NS * 16) +
+                             (piece[k] + shift) * bytes[k];
+    }
+    int st = -1;
+    uint32_t ph = 1;
     for (int t = 0; t < ntile; ++t) {
-      const int st = t % nst, ph = t / nst;
-      if (t >= nst && !tc::mbar_wait(&empty[st], (ph - 1) & 1)) {
+      if (++st == nst) {
+        st = 0;
+        ph ^= 1u;
+      }
+      if (t >= nst && !tc::mbar_wait(&empty[st], ph)) {
         lost = true;
         break;
       }
-      if (lane == 0) tc::mbar_expect(&full[st], pieceb * (uint32_t)nc);
+      if (warp == 16 && lane == 0) tc::mbar_expect(&full[st], pieceb * (uint32_t)nc);
       __syncwarp();
       const uint32_t stage = sbase + (uint32_t)(st * ar.stage_bytes);
-      for (int i = lane; i < ncopy; i += 32) {
-        const int u = i / nc, c = i - u * nc;
-        const long piece = pb + (long)t * nc + c;
-        const int nb = csub[u].nb, bytes = csub[u].bytes;
-        const unsigned char* src = ar.zero;
-        if (piece < pe) {
-          long from = piece;
-          bool ok = true;
-          if (nb != 0) {
-            const unsigned cell = (unsigned)piece / (unsigned)ar.parts;
-            if (nb < 8) {
-              const int ax = (nb - 1) >> 1, up = (nb - 1) & 1;
-              const int idx = (int)((cell / (unsigned)ar.cstr[ax]) % (unsigned)ar.ext[ax]);
-              ok = up ? idx < ar.ext[ax] - 1 : idx > 0;
-              from += (up ? 1L : -1L) * ar.cstr[ax] * ar.parts;
-            } else {
-              const int face = ar.face[nb - 8], ax = face >> 1;
-              const int idx = (int)((cell / (unsigned)ar.cstr[ax]) % (unsigned)ar.ext[ax]);
-              ok = (face & 1) ? idx == ar.ext[ax] - 1 : idx == 0;
-              from = (long)(nb - 8) * ar.parts + (piece - (long)cell * ar.parts);
-            }
+#pragma unroll
+      for (int k = 0; k < kPer; ++k) {
+        if (first + 32 * kXgCopy * k >= ncopy) continue;
+        const bool low_ = idx[k] == 0, up_ = idx[k] == ex[k] - 1;
+        const bool ok = piece[k] < pe && (kind[k] == 0 || (kind[k] == 1 && !low_) || (kind[k] == 2 && !up_) ||
+                                          (kind[k] == 3 && low_) || (kind[k] == 4 && up_));
+        const unsigned char* from = kind[k] >= 3 ? src[k] + (size_t)cpart[k] * bytes[k] : src[k];
+        tc::bulk_g2s(stage + dst[k], ok ? from : ar.zero, (uint32_t)bytes[k], &full[st]);
+        piece[k] += nc;
+        if (kind[k] < 3) src[k] += (long)nc * bytes[k];
+        cpart[k] += nc;
+        while (cpart[k] >= ar.parts) {
+          cpart[k] -= ar.parts;
+          if (++low[k] == cs[k]) {
+            low[k] = 0;
+            if (++idx[k] == ex[k]) idx[k] = 0;
           }
-          if (ok)
-            src = nb >= 8 ? ar.bc + from * bytes
-                          : (csub[u].arr ? ar.dig[1] : ar.dig[0]) +
-                                (size_t)csub[u].c0 * ar.npiece * (ar.po * NS * 16) + from * bytes;
         }
-        tc::bulk_g2s(stage + (uint32_t)c * pieceb + csub[u].dst, src, (uint32_t)bytes, &full[st]);
       }
     }
     // the copies in flight land before the CTA ends (their stages were all consumed otherwise)
@@ -722,49 +751,79 @@ __global__ void __launch_bounds__(kXgThreads, 1)
   } else if (lane == 0) {
     // ---- MMAs
     // K steps of two octets; pieces of 1, 2, 3 or 4 steps (3 and 4: one piece a stage)
-    const int pk = ar.po / 2, ksteps = nc * pk, psh = pk < 3 ? pk - 1 : 2;
-    int folds[kXgGroups] = {0, 0};        // chunks ended so far
+    // (operands in registers, and everything a stage does not change formed before: with them read and computed
+    // between the MMAs a stage took some 1,900 cycles, of 1,024 for its eight MMAs)
+    const int pk = ar.po / 2, ksteps = nc * pk;
+    uint32_t ko[4];
+#pragma unroll
+    for (int kk = 0; kk < 4; ++kk) {
+      const int c = kk / pk;
+      ko[kk] = ((uint32_t)c * pieceb + (uint32_t)(kk - c * pk) * 256u) >> 4;
+    }
+    uint64_t ga[kXgGroups], gb[kXgGroups];
+    uint32_t gi[kXgGroups];
+#pragma unroll
+    for (int g = 0; g < kXgGroups; ++g) {
+      ga[g] = ginfo[g < ng ? g : 0].a;
+      gb[g] = ginfo[g < ng ? g : 0].b;
+      gi[g] = ginfo[g < ng ? g : 0].idesc;
+    }
+    const uint32_t sstep = (uint32_t)(ar.stage_bytes >> 4);
+    uint32_t folds[kXgGroups] = {0, 0};   // chunks ended so far
     bool fresh[kXgGroups] = {true, true}; // the next MMA of the group starts a chunk
+    auto issue = [&](int g, uint64_t da, uint64_t db, uint32_t idesc, uint32_t so, bool start) {
+      const uint32_t d = tmem + (uint32_t)(g * 256);
+      da += so;
+      db += so;
+      tc::mma_f16(d, da + ko[0], db + ko[0], idesc, start ? 0u : 1u);
+      if (ksteps > 1) tc::mma_f16(d, da + ko[1], db + ko[1], idesc, 1u);
+      if (ksteps > 2) tc::mma_f16(d, da + ko[2], db + ko[2], idesc, 1u);
+      if (ksteps > 3) tc::mma_f16(d, da + ko[3], db + ko[3], idesc, 1u);
+    };
+    auto ready = [&](int g, uint32_t done) {  // the accumulators of group g have been folded
+      const bool ok = tc::mbar_wait(&acc_empty[g], (done - 1) & 1);
+      tc::fence_after_sync();
+      return ok;
+    };
+    int st = -1;
+    uint32_t ph = 0, so = 0;
     for (int t = 0; t < ntile; ++t) {
-      const int st = t % nst;
-      if (!tc::mbar_wait(&full[st], (t / nst) & 1)) {
+      if (++st == nst) {
+        st = 0;
+        ph ^= 1u;
+        so = 0;
+      }
+      if (!tc::mbar_wait(&full[st], ph)) {
         lost = true;
         break;
       }
       tc::fence_after_sync();
-      const uint32_t so = (uint32_t)(st * ar.stage_bytes) >> 4;
       // a group whose accumulators are being folded comes last
-      const bool swap = fresh[0] && folds[0] > 0;
-#pragma unroll
-      for (int i = 0; i < kXgGroups; ++i) {
-        const int g = swap ? 1 - i : i;
-        if (g >= ng || lost) continue;
-        const bool start = g == 0 ? fresh[0] : fresh[1];
-        const int done = g == 0 ? folds[0] : folds[1];
-        if (start && done > 0) {
-          if (!tc::mbar_wait(&acc_empty[g], (done - 1) & 1)) lost = true;
-          tc::fence_after_sync();
-          if (lost) continue;
-        }
-        const uint64_t da = ginfo[g].a + so, db = ginfo[g].b + so;
-        const uint32_t idesc = ginfo[g].idesc, d = tmem + (uint32_t)(g * 256);
-#pragma unroll
-        for (int kk = 0; kk < 4; ++kk) {
-          if (kk >= ksteps) break;
-          const int c = kk >> psh;
-          const uint32_t k = ((uint32_t)c * pieceb + (uint32_t)(kk - c * pk) * 256u) >> 4;
-          tc::mma_f16(d, da + k, db + k, idesc, (start && kk == 0) ? 0u : 1u);
-        }
-        const bool ends = xg_ends(g, t, ntile);
-        if (ends) tc::mma_commit(&acc_full[g]);
-        if (g == 0) {
-          fresh[0] = ends;
-          folds[0] += ends;
-        } else {
-          fresh[1] = ends;
-          folds[1] += ends;
-        }
+      const bool swap = ng > 1 && fresh[0] && folds[0] > 0;
+      const bool e0 = xg_ends(0, t, ntile), e1 = xg_ends(1, t, ntile);
+      if (!swap) {
+        if (fresh[0] && folds[0] > 0 && !ready(0, folds[0])) lost = true;
+        if (lost) break;
+        issue(0, ga[0], gb[0], gi[0], so, fresh[0]);
+        if (e0) tc::mma_commit(&acc_full[0]);
       }
+      if (ng > 1) {
+        if (fresh[1] && folds[1] > 0 && !ready(1, folds[1])) lost = true;
+        if (lost) break;
+        issue(1, ga[1], gb[1], gi[1], so, fresh[1]);
+        if (e1) tc::mma_commit(&acc_full[1]);
+        fresh[1] = e1;
+        folds[1] += e1;
+      }
+      if (swap) {
+        if (!ready(0, folds[0])) lost = true;
+        if (lost) break;
+        issue(0, ga[0], gb[0], gi[0], so, true);
+        if (e0) tc::mma_commit(&acc_full[0]);
+      }
+      fresh[0] = e0;
+      folds[0] += e0;
+      so += sstep;
       if (lost) break;
       tc::mma_commit(&empty[st]);
     }
@@ -1072,8 +1131,8 @@ tt_status xg_launch_products(cudaStream_t s, const XgPlan& pl, XgArgs& args, lon
                              int ldg, size_t plane, unsigned long long* gint, const unsigned long long* slots, int* unit,
                              double* coef, int* status) {
   constexpr int W = XgCfg<NS>::W;
-  args.stage_bytes = xg_stage_bytes(pl);
-  args.nstage = xg_stages(pl);
+  args.stage_bytes = xg_stage_bytes(pl, args.nc * args.po);
+  args.nstage = xg_stages(pl, args.nc * args.po);
   size_t smem = args.stage_bytes * args.nstage + kXgPad;
   if (smem < 117 * 1024) smem = 117 * 1024;  // one CTA per SM: its accumulators never wait for another's
   auto kern = k_xg_mma<NS>;
@@ -1124,7 +1183,7 @@ tt_status xg_factor(cudaStream_t s, int num_sms, int sms, const Src& src, LivePa
   if (!bc) nbc = 0;
   args.po = ar.po;
   args.parts = ar.parts;
-  args.nc = 8 / ar.po;
+  args.nc = kXgStageOct / ar.po;
   args.npiece = ar.npiece;
   long groups;
   xg_groups(args.npiece, args.nc, pl.ncta, sms > 0 ? sms : num_sms, groups, args.ppg);
