@@ -1,11 +1,13 @@
 // Gram-based factor of the merged core (the Gram method among the paper's rounding methods,
-// Sec. 3.1): G = A^T A of the (possibly virtual) N_Z x R matrix A in FP64, then a square root
+// Sec. 3.1): G = A^T A of the (possibly virtual) N_Z x R matrix A, from the exact products (xgram.cuh) rounded
+// once to FP64, or in FP64 tiles where the workspace cannot hold their digits; then a square root
 // R of G (R^T R = G, from a diagonally pivoted Cholesky), which stands in for the TSQR's R factor
 // (the small-core sweep uses R only through R^T R).  Forming G squares the condition
 // number: singular values below about sqrt(eps) |A| are not resolved.
 #pragma once
 #include "bigpass.cuh"
 #include "small.cuh"
+#include "xgram.cuh"
 
 namespace ttk {
 
@@ -232,11 +234,12 @@ tt_status gram_matrix(cudaStream_t s, int num_sms, const Src& src, LivePattern l
 // Takes its workspace from `ws` in dry runs too (same order), launches nothing then.
 template <class Src>
 tt_status gram_factor(cudaStream_t s, int num_sms, const Src& src, LivePattern lp, long nrows, Bump& ws,
-                      DevCtrl* ctrl, int coop_grid_max, double** RZ_out, int timer_cat = kTsqrLeaf) {
+                      DevCtrl* ctrl, int sms, bool exact, double** RZ_out, int timer_cat = kTsqrLeaf) {
   const int ncap = lp.ncap();
   if (ncap > 512) return TT_ERR_UNSUPPORTED;
   double* G = nullptr;
-  tt_status st = gram_matrix(s, num_sms, src, lp, nrows, ws, &G, timer_cat);
+  tt_status st = exact ? xg_factor<double>(s, num_sms, sms, src, lp, nrows, ws, &G, &ctrl->status, timer_cat, true)
+                       : gram_matrix(s, num_sms, src, lp, nrows, ws, &G, timer_cat);
   if (st != TT_OK) return st;
   int* perm = ws.take<int>(ncap);
   double* RZ = ws.take<double>((size_t)ncap * ncap);

@@ -299,6 +299,11 @@ template <typename T, class Src>
 inline bool xg_takes(const tt_context* ctx, const TsqrCfg& cfg, const Src& src, const LivePattern& lp, long nrows) {
   return !cfg.set && !ctx->no_xg && xg_fits<T>(src, lp, nrows);
 }
+// Whether Gram-SVD rounding takes its Gram matrix from them.
+template <class Src>
+inline bool xg_gram(const tt_context* ctx, const Src& src, const LivePattern& lp, long nrows) {
+  return !ctx->no_xg && xg_fits<double>(src, lp, nrows);
+}
 // SMs such a pass may take: all of them, or a batched problem's share (its leaf cap).
 template <typename T>
 inline int xg_sms(const tt_context* ctx) {
@@ -454,8 +459,8 @@ tt_status round_impl(tt_context* ctx, tt_tensor* x, double tol, int rmax, Bump& 
     cudaMemsetAsync(domega_ones, 0, sizeof(double) * (size_t)n1 * n2, s);
   }
   if (ctx->rounding == TT_ROUND_GRAM) {
-    tt_status st = gram_factor(s, ctx->num_sms, SrcRows<S>{(const S*)x->core[0], K1}, lp, N, ws, ctx->ctrl,
-                               ctx->coop_grid_max, &RZ);
+    tt_status st = gram_factor(s, ctx->num_sms, src, lp, N, ws, ctx->ctrl, xg_sms<T>(ctx), xg_gram(ctx, src, lp, N),
+                               &RZ);
     if (st != TT_OK) return st;
   } else if (ctx->rounding == TT_ROUND_RANDOMIZED) {
     tt_status st = randomized_factor<S, T>(ctx, s, SrcRows<S>{(const S*)x->core[0], K1}, lp, N, b.Bbase, n1 * n2, ws,
@@ -548,7 +553,8 @@ tt_status step_impl(tt_context* ctx, const tt_plan* p, tt_tensor* I, double tol,
   const bool gram = (ctx->rounding == TT_ROUND_GRAM);
   const bool rnd = (ctx->rounding == TT_ROUND_RANDOMIZED);
   if (gram) {
-    tt_status st = gram_factor(s, ctx->num_sms, src1, lp1, N, ws, ctx->ctrl, ctx->coop_grid_max, &RZ1);
+    tt_status st = gram_factor(s, ctx->num_sms, src1, lp1, N, ws, ctx->ctrl, xg_sms<T>(ctx),
+                               xg_gram(ctx, src1, lp1, N), &RZ1);
     if (st != TT_OK) return st;
   } else if (rnd) {
     tt_status st = randomized_factor<S, T>(ctx, s, src1, lp1, N, b1.B0, nang, ws, &RZ1, kTsqrLeaf);
@@ -584,7 +590,8 @@ tt_status step_impl(tt_context* ctx, const tt_plan* p, tt_tensor* I, double tol,
     (void)take_ud<T>(ctx, SrcRows<S>{Zsrc, K1 + 1}, lp2, N, K1, ws, ub2);
     if (gram) {
       double* RZ2 = nullptr;
-      st = gram_factor(s, ctx->num_sms, SrcRows<S>{Zsrc, K1 + 1}, lp2, N, ws, ctx->ctrl, ctx->coop_grid_max, &RZ2);
+      st = gram_factor(s, ctx->num_sms, SrcRows<S>{Zsrc, K1 + 1}, lp2, N, ws, ctx->ctrl, xg_sms<T>(ctx),
+                       xg_gram(ctx, SrcRows<S>{Zsrc, K1 + 1}, lp2, N), &RZ2);
       if (st != TT_OK) return st;
     } else if (rnd) {
       double* RZ2 = nullptr;
@@ -618,8 +625,8 @@ tt_status step_impl(tt_context* ctx, const tt_plan* p, tt_tensor* I, double tol,
   k_b0_source<<<64, 256, 0, s>>>(K1, nang, b1.Bnew, b2.B0); count_launch();
   double* RZ2 = nullptr;
   if (gram)
-    st = gram_factor(s, ctx->num_sms, SrcRows<S>{Zsrc, K1 + 1}, lp2, N, ws, ctx->ctrl, ctx->coop_grid_max, &RZ2,
-                     kTsqrLeafSrc);
+    st = gram_factor(s, ctx->num_sms, SrcRows<S>{Zsrc, K1 + 1}, lp2, N, ws, ctx->ctrl, xg_sms<T>(ctx),
+                     xg_gram(ctx, SrcRows<S>{Zsrc, K1 + 1}, lp2, N), &RZ2, kTsqrLeafSrc);
   else if (rnd)
     st = randomized_factor<S, T>(ctx, s, SrcRows<S>{Zsrc, K1 + 1}, lp2, N, b2.B0, nang, ws, &RZ2, kTsqrLeafSrc);
   else if (xg2)

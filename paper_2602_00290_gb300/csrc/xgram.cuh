@@ -1182,12 +1182,66 @@ void xg_launch_digits(cudaStream_t s, int num_sms, const S* A, const XgArray& ar
   count_launch();
 }
 
+// 192-bit integer times 2^e, rounded.
+__device__ __forceinline__ double real192(Int192 g, int e) {
+  const bool neg = (long long)g.w[2] < 0;
+  if (neg) {
+    const Int192 one{{1ull, 0ull, 0ull}};
+    g = Int192{{~g.w[0], ~g.w[1], ~g.w[2]}};
+    add192(g, one.w[0], one.w[1], one.w[2]);
+  }
+  // the top 64 bits and a sticky bit
+  int up = 128;
+  unsigned long long hi = g.w[2], mid = g.w[1], lo = g.w[0];
+  if (hi == 0ull) {
+    hi = mid;
+    mid = lo;
+    lo = 0ull;
+    up = 64;
+  }
+  if (hi == 0ull) {
+    hi = mid;
+    mid = 0ull;
+    up = 0;
+  }
+  if (hi == 0ull) return 0.0;
+  const int lz = __clzll((long long)hi);
+  unsigned long long top = lz ? (hi << lz) | (mid >> (64 - lz)) : hi;
+  const unsigned long long rest = lz ? (mid << lz) | (lo >> (64 - lz)) : (mid | lo);
+  if (rest | lo) top |= 1ull;
+  const double v = ldexp(__ull2double_rn(top), up - lz + e);
+  return neg ? -v : v;
+}
+// Gram matrix in FP64 from its integers (upper triangle), units and coefficients applied.
+template <int NS>
+__global__ void __launch_bounds__(256) k_xg_real(int n, const unsigned long long* __restrict__ gint,
+                                                 const int* __restrict__ unit, const double* __restrict__ coef,
+                                                 double* __restrict__ out) {
+  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (i >= n * n) return;
+  const int a = i / n, b = i - a * n;
+  const size_t plane = (size_t)n * n, o = a <= b ? i : (size_t)b * n + a;
+  const Int192 g{{gint[o], gint[plane + o], gint[2 * plane + o]}};
+  out[i] = coef[a] * coef[b] * real192(g, unit[a] + unit[b]);
+}
+template <int NS>
+__global__ void __launch_bounds__(256) k_xg_real_cols(int rows, int cols, size_t plane, const unsigned long long* __restrict__ gint,
+                                                      const unsigned long long* __restrict__ sa,
+                                                      const unsigned long long* __restrict__ sb, double* __restrict__ out) {
+  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (i >= rows * cols) return;
+  const int a = i / cols, b = i - a * cols;
+  const Int192 g{{gint[i], gint[plane + i], gint[2 * plane + i]}};
+  out[i] = real192(g, xg_unit(sa[a], NS) + xg_unit(sb[b], NS));
+}
+
 // Triangular factor RZ (ncap x ncap, row-major; R^T R = A^T A) of the source's columns.  sms: SMs this
 // pass may take.  Dry runs take the workspace only; everything but RZ is released on return (later
 // work on the stream may overwrite it).
+// gram: R is the Gram matrix itself instead.
 template <typename T, class Src>
 tt_status xg_factor(cudaStream_t s, int num_sms, int sms, const Src& src, LivePattern lp, long nrows, Bump& ws,
-                    double** RZ_out, int* status, int leaf_cat = kTsqrLeaf) {
+                    double** RZ_out, int* status, int leaf_cat = kTsqrLeaf, bool gram = false) {
   using S = typename XgElem<Src>::type;
   constexpr int NS = sizeof(T) == 4 ? 4 : 8;
   constexpr int W = XgCfg<NS>::W, H = XgCfg<NS>::H;
@@ -1247,6 +1301,11 @@ tt_status xg_factor(cudaStream_t s, int num_sms, int sms, const Src& src, LivePa
       k_xg_combine<NS, Src><<<(unsigned)((n * n + 255) / 256), 256, 0, s>>>(src, n, pl.nraw, raw, slots, gint, unit, coef);
       count_launch();
     }
+  }
+  if (gram) {
+    k_xg_real<NS><<<(unsigned)((n * n + 255) / 256), 256, 0, s>>>(n, gint, unit, coef, R);
+    count_launch();
+    return cudaGetLastError() == cudaSuccess ? TT_OK : TT_ERR_CUDA;
   }
   TimerScope scope(kTsqrMerge, s);
   return launch_xg_chol<(NS == 4 ? 1 : 2)>(s, n, gint, unit, coef, R);
