@@ -2,6 +2,7 @@
 #include "bigpass.cuh"
 #include "small.cuh"
 #include "step.cuh"
+#include "xgram.cuh"
 
 namespace ttk {
 namespace {
@@ -170,10 +171,12 @@ __global__ void k_axpy_ranks(int d, const int* __restrict__ rx, int* __restrict_
   if (d == 3) ry[2] = n2;
 }
 
-// Per-chunk partial Gram entries W1[a][b] = sum_k X[k][a] Y[k][b].
+// Per-chunk partial Gram entries W1[a][b] = sum_k X[k][a] Y[k][b]; when (nullable): a no-op where it is zero.
 template <typename S>
 __global__ void k_gram_partials(long N, long rows_per, const S* __restrict__ X, int ldx, int rx,
-                                const S* __restrict__ Y, int ldy, int ry, double* __restrict__ partials) {
+                                const S* __restrict__ Y, int ldy, int ry, double* __restrict__ partials,
+                                const int* __restrict__ when) {
+  if (when && *when == 0) return;
   const int e = blockIdx.y * blockDim.x + threadIdx.x;
   if (e >= rx * ry) return;
   const int a = e / ry, b = e - (e / ry) * ry;
@@ -184,7 +187,9 @@ __global__ void k_gram_partials(long N, long rows_per, const S* __restrict__ X, 
   partials[(size_t)blockIdx.x * rx * ry + e] = acc;
 }
 
-__global__ void k_sum_chunks(const double* __restrict__ partials, long nchunks, int ne, double* __restrict__ out) {
+__global__ void k_sum_chunks(const double* __restrict__ partials, long nchunks, int ne, double* __restrict__ out,
+                             const int* __restrict__ when) {
+  if (when && *when == 0) return;
   const int e = blockIdx.x * blockDim.x + threadIdx.x;
   if (e >= ne) return;
   double s = 0.0;
@@ -253,6 +258,7 @@ tt_status axpy_impl(tt_context* ctx, double alpha, const tt_tensor* x, tt_tensor
   return cudaGetLastError() == cudaSuccess ? TT_OK : TT_ERR_CUDA;
 }
 
+constexpr long kDotExactRows = 16384;
 template <typename S>
 tt_status dot_impl(tt_context* ctx, const tt_tensor* x, const tt_tensor* y, double* out, Bump& ws) {
   cudaStream_t s = ctx->stream;
@@ -270,11 +276,20 @@ tt_status dot_impl(tt_context* ctx, const tt_tensor* x, const tt_tensor* y, doub
   double* Bx = ws.take<double>((size_t)rx * nang);
   double* By = ws.take<double>((size_t)ry * nang);
   double* G = ws.take<double>(ne);
+  // tall cores: exact products on the tensor cores, the FP64 sums only where an entry is not finite.  From 16,384
+  // rows on; fewer are a few microseconds either way
+  const XgPair<S> pr{(const S*)x->core[0], (const S*)y->core[0], rx, ry};
+  int* when = nullptr;
+  if (!ctx->no_xg && N >= kDotExactRows && xg_cross_fits(pr)) {
+    when = ws.take<int>(1);
+    const tt_status st = xg_cross<S>(s, ctx->num_sms, pr, N, ws, W1, when, &ctx->ctrl->status);
+    if (st != TT_OK) return st;
+  }
   if (ws.dry) return TT_OK;
   dim3 grid((unsigned)nchunks, (unsigned)((ne + 255) / 256));
   k_gram_partials<S><<<grid, 256, 0, s>>>(N, rows_per, (const S*)x->core[0], rx, rx, (const S*)y->core[0], ry, ry,
-                                          part); count_launch();
-  k_sum_chunks<<<(ne + 255) / 256, 256, 0, s>>>(part, nchunks, ne, W1); count_launch();
+                                          part, when); count_launch();
+  k_sum_chunks<<<(ne + 255) / 256, 256, 0, s>>>(part, nchunks, ne, W1, when); count_launch();
   right_part<S>(s, d, rx, n1, d == 3 ? x->rcap[2] : 1, n2, (const S*)x->core[1], d == 3 ? (const S*)x->core[2] : nullptr,
                 Bx);
   right_part<S>(s, d, ry, n1, d == 3 ? y->rcap[2] : 1, n2, (const S*)y->core[1], d == 3 ? (const S*)y->core[2] : nullptr,
@@ -310,8 +325,8 @@ tt_status dot_into(cudaStream_t s, const tt_tensor* x, const tt_tensor* y, doubl
   double* G = By + (size_t)ry * nang;
   dim3 grid((unsigned)nchunks, (unsigned)((ne + 255) / 256));
   k_gram_partials<S><<<grid, 256, 0, s>>>(N, rows_per, (const S*)x->core[0], rx, rx, (const S*)y->core[0], ry, ry,
-                                          part); count_launch();
-  k_sum_chunks<<<(unsigned)((ne + 255) / 256), 256, 0, s>>>(part, nchunks, (int)ne, W1); count_launch();
+                                          part, nullptr); count_launch();
+  k_sum_chunks<<<(unsigned)((ne + 255) / 256), 256, 0, s>>>(part, nchunks, (int)ne, W1, nullptr); count_launch();
   right_part<S>(s, d, rx, n1, d == 3 ? x->rcap[2] : 1, n2, (const S*)x->core[1], d == 3 ? (const S*)x->core[2] : nullptr,
                 Bx);
   right_part<S>(s, d, ry, n1, d == 3 ? y->rcap[2] : 1, n2, (const S*)y->core[1], d == 3 ? (const S*)y->core[2] : nullptr,

@@ -1310,4 +1310,105 @@ tt_status xg_factor(cudaStream_t s, int num_sms, int sms, const Src& src, LivePa
   TimerScope scope(kTsqrMerge, s);
   return launch_xg_chol<(NS == 4 ? 1 : 2)>(s, n, gint, unit, coef, R);
 }
+
+// Products of the columns of two matrices over the same rows (explicit rows, FP64 digits).
+template <typename S>
+struct XgPair {
+  const S *A, *B;
+  int na, nb;
+};
+template <typename S>
+struct XgElem<XgPair<S>> { using type = S; static constexpr bool stencil = false; };
+template <int NS, typename S>
+inline bool xg_make_plan(const XgPair<S>& s, const LivePattern&, XgPlan& pl) {
+  pl.nsub = 0;
+  pl.nraw = s.na + s.nb;
+  return s.na <= 256 && s.nb <= 256 && xg_add<NS>(pl, s.na, 0, 0, 0) && xg_add<NS>(pl, s.nb, s.na, 1, 0) &&
+         xg_tiles<NS>(pl, true) && xg_stages(pl) >= 2;
+}
+template <typename S>
+inline long xg_plan_key(const XgPair<S>& s, const LivePattern&) { return 1000L * s.na + s.nb; }
+
+// Rows per pass of xg_cross: the workspace (256 MB of digits at 2 x 32 columns) does not grow with the rows;
+// 65,536 rows a pass spent half of the time in k_xg_sum.
+constexpr long kXgCrossRows = 1L << 18;
+template <typename S>
+inline const XgPlan* xg_cross_plan(const XgPair<S>& pr) {
+  // a matrix with itself: the upper triangle
+  if (pr.A == pr.B && pr.na == pr.nb) return xg_plan_of<8>(SrcRows<S>{pr.A, pr.na}, LivePattern{nullptr, pr.na, 1, 0});
+  return xg_plan_of<8>(pr, LivePattern{nullptr, 1, 1, 0});
+}
+template <typename S>
+inline bool xg_cross_fits(const XgPair<S>& pr) { return xg_cross_plan(pr) != nullptr; }
+
+// W (na x nb, row-major) = A^T B of two row-major matrices, from exact products of their columns' fixed
+// points; *nonfinite is set (or cleared) for an Inf or NaN, and W is then to be formed otherwise.  An entry's
+// error is its columns' rounding, 2^-62 of their largest entries: an FP64 sum rounds by 2^-53 of its
+// terms, and ran at the rate of the FP64 pipe: three products of 1,048,576 x 32 x 32 columns 6.5 ms, now 2.0.
+template <typename S>
+tt_status xg_cross(cudaStream_t s, int num_sms, const XgPair<S>& pr, long nrows, Bump& ws, double* W, int* nonfinite,
+                   int* status) {
+  constexpr int NS = 8, H = XgCfg<NS>::H, Wd = XgCfg<NS>::W;
+  const LivePattern la{nullptr, pr.na, 1, 0}, lb{nullptr, pr.nb, 1, 0};
+  const XgPlan& pl = *xg_cross_plan(pr);
+  const int nmat = pr.A == pr.B && pr.na == pr.nb ? 1 : 2;
+  const long rows = nrows < kXgCrossRows ? nrows : kXgCrossRows;
+  XgArray aa, ab;
+  const S* p = nullptr;
+  if (!xg_array(SrcRows<S>{pr.A, pr.na}, pr.na, rows, aa, &p) || !xg_array(SrcRows<S>{pr.B, pr.nb}, pr.nb, rows, ab, &p))
+    return TT_ERR_UNSUPPORTED;
+  const size_t mark = ws.off;
+  const int n = pr.na + pr.nb;
+  const size_t zbytes = (size_t)8 * NS * Wd * 16, plane = (size_t)pr.na * pr.nb;
+  unsigned char* zeroed = ws.take<unsigned char>(zbytes + 8 * (size_t)n);
+  unsigned long long* slots = reinterpret_cast<unsigned long long*>(zeroed + zbytes);
+  unsigned char* da = ws.take<unsigned char>((size_t)aa.npiece * aa.po * aa.cpad * (NS * 16));
+  unsigned char* db = nmat == 1 ? da : ws.take<unsigned char>((size_t)ab.npiece * ab.po * ab.cpad * (NS * 16));
+  unsigned long long* gint = ws.take<unsigned long long>(3 * plane);
+  XgArgs args{};
+  args.po = aa.po;
+  args.parts = aa.parts;
+  args.nc = kXgStageOct / aa.po;
+  args.npiece = aa.npiece;
+  long groups;
+  xg_groups(args.npiece, args.nc, pl.ncta, num_sms, groups, args.ppg);
+  long long* part = ws.take<long long>((size_t)groups * pl.ncta * kXgTiles * (H * Wd * 128));
+  ws.release(mark);
+  if (ws.dry) return TT_OK;
+  cudaMemsetAsync(zeroed, 0, zbytes + 8 * (size_t)n, s);
+  cudaMemsetAsync(nonfinite, 0, sizeof(int), s);
+  for (int i = 0; i < nmat; ++i) {
+    const XgArray& ar = i ? ab : aa;
+    const long rpb = 256 / ar.ncol, need = (nrows + 8 * rpb - 1) / (8 * rpb);
+    const long grid = need < 8L * num_sms ? need : 8L * num_sms;
+    k_xg_colmax<S><<<(unsigned)(grid > 0 ? grid : 1), 256, 0, s>>>(i ? pr.B : pr.A, ar.ncol, ar.sr, ar.sc, nrows,
+                                                                   slots + (i ? pr.na : 0), nullptr, 0, ar.G, nonfinite);
+    count_launch();
+  }
+  args.dig[0] = da;
+  args.dig[1] = db;
+  args.bc = nullptr;
+  args.zero = zeroed;
+  for (long r0 = 0; r0 < nrows; r0 += rows) {
+    const long m = nrows - r0 < rows ? nrows - r0 : rows;
+    for (int i = 0; i < nmat; ++i) {
+      const XgArray& ar = i ? ab : aa;
+      const long tot = ar.npiece * ar.po * ar.cpad;
+      long grid = (tot + 255) / 256;
+      if (grid > 16L * num_sms) grid = 16L * num_sms;
+      // rows past m: zero digits
+      k_xg_digits<NS, S><<<(unsigned)grid, 256, 0, s>>>((i ? pr.B : pr.A) + r0 * ar.sr, ar, i ? lb : la, m,
+                                                        slots + (i ? pr.na : 0), i ? db : da, nullptr, 0, nullptr);
+      count_launch();
+    }
+    const tt_status st = xg_launch_products<NS>(s, pl, args, groups, part, nmat == 1 ? 0 : pr.na, pr.nb, plane, gint, slots,
+                                                nullptr, nullptr,
+                                                status, r0 > 0);
+    if (st != TT_OK) return st;
+  }
+  k_xg_real_cols<NS><<<(unsigned)((plane + 255) / 256), 256, 0, s>>>(pr.na, pr.nb, plane, gint, slots,
+                                                                       slots + (nmat == 1 ? 0 : pr.na), W);
+  count_launch();
+  return cudaGetLastError() == cudaSuccess ? TT_OK : TT_ERR_CUDA;
+}
 }  // namespace ttk
