@@ -147,6 +147,49 @@ __global__ void k_rowdot_partials(long nrows, int ld, int ncol, const S* __restr
   if (threadIdx.x == 0 && partials) partials[blockIdx.x] = s;
 }
 
+// x in FP64 on the integer units (the conversion runs on the FP64 pipe, 1/64 of the FP32 rate).
+__device__ __forceinline__ double widen(float x) {
+  const unsigned b = __float_as_uint(x), e = (b >> 23) & 0xffu;
+  if (e - 1u >= 254u) return (double)x;
+  return __hiloint2double((int)((b & 0x80000000u) | (((b & 0x7fffffffu) >> 3) + (896u << 20))), (int)(b << 29));
+}
+__device__ __forceinline__ double widen(double x) { return x; }
+
+// partials[cta] = sum over the CTA's rows of Z[k,:] . v, as v . (column sums): a thread keeps one column (whole
+// rows per warp, one FP64 addition an entry).  A thread per row (k_rowdot_partials) read a sector per entry:
+// 1.32 ms at 3,538,944 rows x 48 FP32.
+template <typename S>
+__global__ void __launch_bounds__(256) k_colsum_dot(long nrows, int ld, int ncol, const S* __restrict__ Z,
+                                                    const double* __restrict__ v, double* __restrict__ partials) {
+  __shared__ double red[256];
+  const int tid = threadIdx.x, rpb = 256 / ncol, sub = tid / ncol, q = tid - sub * ncol;
+  double a0 = 0.0, a1 = 0.0;
+  if (sub < rpb) {
+    const long per = (nrows + gridDim.x - 1) / gridDim.x, beg = per * blockIdx.x;
+    const long end = beg + per < nrows ? beg + per : nrows;
+    long k = beg + sub;
+    for (; k + 7 * rpb < end; k += 8 * rpb) {
+      S x[8];
+#pragma unroll
+      for (int u = 0; u < 8; ++u) x[u] = Z[(k + u * rpb) * ld + q];
+#pragma unroll
+      for (int u = 0; u < 8; u += 2) {
+        a0 += widen(x[u]);
+        a1 += widen(x[u + 1]);
+      }
+    }
+    for (; k < end; k += rpb) a0 += widen(Z[k * ld + q]);
+    a0 = (a0 + a1) * v[q];
+  }
+  red[tid] = a0;
+  __syncthreads();
+  for (int o = 128; o; o >>= 1) {
+    if (tid < o) red[tid] += red[tid + o];
+    __syncthreads();
+  }
+  if (tid == 0) partials[blockIdx.x] = red[0];
+}
+
 __global__ void k_energy_pack(const double* __restrict__ e_before, const double* __restrict__ e1,
                               const double* __restrict__ e2, double scale, double* __restrict__ out) {
   if (threadIdx.x == 0 && blockIdx.x == 0) {
@@ -216,8 +259,8 @@ static tt_status launch_update_blk(cudaStream_t s, int num_sms, const SrcStencil
   return cudaGetLastError() == cudaSuccess ? TT_OK : TT_ERR_CUDA;
 }
 
-// The update pass of a rounding: the tensor-core kernel (ctx->tensor_cores, FP32 storage of the
-// stencil source) where it takes the pass, else the FP32 kernel over staged row blocks, else the
+// The update pass of a rounding: from digits where its buffers were taken (take_ud), the split-TF32 kernel
+// (ctx->tensor_cores, FP32 storage of the stencil source) where it takes the pass, else the FP32 kernel over staged row blocks, else the
 // generic kernel.
 template <typename T, class Src, class Epi>
 static tt_status launch_update(const tt_context* ctx, cudaStream_t s, int num_sms, const Src& src, LivePattern lp,
@@ -543,9 +586,15 @@ tt_status step_impl(tt_context* ctx, const tt_plan* p, tt_tensor* I, double tol,
     right_part<S>(s, d, K1, n1, K2, n2, (const S*)I->core[1], d == 3 ? (const S*)I->core[2] : nullptr, b1.Bbase);
     if (energy) {
       k_vj_host_launch(s, K1, nang, b1.Bbase, p->domega, vJ0);
-      k_rowdot_partials<S><<<(unsigned)((N + 255) / 256), 256, 0, s>>>(N, K1, K1, (const S*)I->core[0], vJ0, part0,
-                                                                      nullptr, 0.0); count_launch();
-      reduce_partials(s, part0, (N + 255) / 256, 1, sums, 1.0);
+      long nb = (N + 255) / 256;
+      if (K1 <= 256) {
+        if (nb > 8L * ctx->num_sms) nb = 8L * ctx->num_sms;
+        k_colsum_dot<S><<<(unsigned)nb, 256, 0, s>>>(N, K1, K1, (const S*)I->core[0], vJ0, part0);
+      } else {
+        k_rowdot_partials<S><<<(unsigned)nb, 256, 0, s>>>(N, K1, K1, (const S*)I->core[0], vJ0, part0, nullptr, 0.0);
+      }
+      count_launch();
+      reduce_partials(s, part0, nb, 1, sums, 1.0);
     }
     k_b0_transport<<<256, 256, 0, s>>>(K1, p->nterm, p->nbc, n1, n2, b1.Bbase, p->fac1, p->fac2, p->bc_term_dev,
                                        b1.B0); count_launch();
