@@ -359,8 +359,8 @@ tt_status dot_impl(tt_context* ctx, const tt_tensor* x, const tt_tensor* y, doub
   double* Bx = ws.take<double>((size_t)rx * nang);
   double* By = ws.take<double>((size_t)ry * nang);
   double* G = ws.take<double>(ne);
-  // tall cores: exact products on the tensor cores, the FP64 sums only where an entry is not finite.  From 16,384
-  // rows on; fewer are a few microseconds either way
+  // tall cores: exact products on the tensor cores, the FP64 sums only where an entry is not finite or the columns
+  // are large on different rows (k_xg_cover).  From 16,384 rows on; fewer are a few microseconds either way
   const XgPair<S> pr{(const S*)x->core[0], (const S*)y->core[0], rx, ry};
   int* when = nullptr;
   if (!ctx->no_xg && N >= kDotExactRows && xg_cross_fits(pr)) {

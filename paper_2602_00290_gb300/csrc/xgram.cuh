@@ -28,6 +28,7 @@
 // FP64 0.28, 1.7 ms (before 99.6 + 14 ms).  With base 512 and MMAs of N = 128 columns over octets copied one by
 // one the products took 0.87 and 3.06 ms.
 #pragma once
+#include <cmath>
 #include <map>
 #include <vector>
 
@@ -1329,6 +1330,75 @@ inline bool xg_make_plan(const XgPair<S>& s, const LivePattern&, XgPlan& pl) {
 template <typename S>
 inline long xg_plan_key(const XgPair<S>& s, const LivePattern&) { return 1000L * s.na + s.nb; }
 
+// Whether the fixed point holds an inner product as well as FP64 sums do.  A column's rounding is 2^-62 of its
+// largest entry, so a product of N rows is off by about 2^-62 sqrt(N) max|a| max|b|, an FP64 sum by 2^-53 of
+// sum |a||b| or more: where the columns are large on different rows (sum |a||b| below 2^-9 sqrt(N) max|a| max|b|),
+// the FP64 sums are the better ones.  sum |a||b| is bounded from below by one row of every `stride` (a hashed one: a
+// fixed one would meet the same group in every cell): a CTA takes 16 x 16 pairs and 64 of these rows at a time, in
+// units of the columns' powers of two; the sums are integers (2^-20), so that the decision does not depend on the
+// order.  About 25 us of a product of 1,048,576 x 32 x 32 columns (0.74 ms in all; 0.72 ms without); with FP64
+// conversions instead of integers and twice the rows 55 us.
+constexpr long kXgCoverRows = 1L << 15;
+__device__ __forceinline__ int xg_cover_exp(unsigned long long slot) { return (int)(slot >> 52); }
+// |x| in units of 2^(ex - 1022), cut to FP32 (integers: the conversion runs on the FP64 pipe); ex: exponent field of
+// the column's largest entry as FP64.
+__device__ __forceinline__ float xg_cover_val(int e, unsigned m23, int ex) {
+  const int f = min(e - ex + 126, 126);
+  return e > 0 && f > 0 ? __uint_as_float(((unsigned)f << 23) | m23) : 0.0f;
+}
+__device__ __forceinline__ float xg_cover_abs(double x, int ex) {
+  const unsigned long long b = (unsigned long long)__double_as_longlong(x);
+  return xg_cover_val((int)((b >> 52) & 0x7ffu), (unsigned)(b >> 29) & 0x7fffffu, ex);
+}
+__device__ __forceinline__ float xg_cover_abs(float x, int ex) {
+  const unsigned b = __float_as_uint(x);
+  return xg_cover_val((int)((b >> 23) & 0xffu), b & 0x7fffffu, ex - 896);
+}
+template <typename S>
+__global__ void __launch_bounds__(256) k_xg_cover(const S* __restrict__ A, const S* __restrict__ B, int na, int nb,
+                                                  long nrows, long stride, const unsigned long long* __restrict__ sa,
+                                                  const unsigned long long* __restrict__ sb,
+                                                  unsigned long long* __restrict__ cover) {
+  __shared__ float va[64][17], vb[64][17];
+  const int ta = (nb + 15) / 16, a0 = (int)blockIdx.y / ta * 16, b0 = (int)blockIdx.y % ta * 16;
+  const int tid = threadIdx.x, ia = tid >> 4, ib = tid & 15;
+  const long nsamp = (nrows + stride - 1) / stride;
+  const bool la = a0 + ib < na, lb = b0 + ib < nb;
+  const int fa = la ? xg_cover_exp(sa[a0 + ib]) : 0, fb = lb ? xg_cover_exp(sb[b0 + ib]) : 0;
+  float sum = 0.0f;
+  for (long m0 = (long)blockIdx.x * 64; m0 < nsamp; m0 += (long)gridDim.x * 64) {
+    __syncthreads();
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      const int m = ia + 16 * u;
+      const long k = (m0 + m) * stride + (long)((((unsigned)(m0 + m) * 2654435761u) >> 8) % (unsigned)stride);
+      const bool in = m0 + m < nsamp && k < nrows;
+      va[m][ib] = in && la ? xg_cover_abs(A[k * na + a0 + ib], fa) : 0.0f;
+      vb[m][ib] = in && lb ? xg_cover_abs(B[k * nb + b0 + ib], fb) : 0.0f;
+    }
+    __syncthreads();
+#pragma unroll 16
+    for (int m = 0; m < 64; ++m) sum = fmaf(va[m][ia], vb[m][ib], sum);
+  }
+  if (a0 + ia < na && lb)
+    atomicAdd(&cover[(size_t)(a0 + ia) * nb + b0 + ib], (unsigned long long)(sum * 1048576.0f));
+}
+// Sets *nonfinite for a pair that is not covered, or whose columns are so small that the storage's subnormal
+// numbers (dropped from the fixed point) would count.
+template <typename S>
+__global__ void __launch_bounds__(256) k_xg_cover_check(int na, int nb, double least,
+                                                        const unsigned long long* __restrict__ sa,
+                                                        const unsigned long long* __restrict__ sb,
+                                                        const unsigned long long* __restrict__ cover,
+                                                        int* __restrict__ nonfinite) {
+  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (i >= na * nb) return;
+  const unsigned long long ma = sa[i / nb], mb = sb[i % nb];
+  if (ma == 0ull || mb == 0ull) return;
+  constexpr int kLow = sizeof(S) == 4 ? 1023 - 63 : 64;
+  if (xg_cover_exp(ma) < kLow || xg_cover_exp(mb) < kLow || (double)cover[i] < least) *nonfinite = 1;
+}
+
 // Rows per pass of xg_cross: the workspace (256 MB of digits at 2 x 32 columns) does not grow with the rows;
 // 65,536 rows a pass spent half of the time in k_xg_sum.
 constexpr long kXgCrossRows = 1L << 18;
@@ -1342,9 +1412,10 @@ template <typename S>
 inline bool xg_cross_fits(const XgPair<S>& pr) { return xg_cross_plan(pr) != nullptr; }
 
 // W (na x nb, row-major) = A^T B of two row-major matrices, from exact products of their columns' fixed
-// points; *nonfinite is set (or cleared) for an Inf or NaN, and W is then to be formed otherwise.  An entry's
+// points; *nonfinite is set (or cleared) for an Inf or NaN and for columns that the fixed point does not hold as well
+// as FP64 sums (k_xg_cover), and W is then to be formed otherwise.  An entry's
 // error is its columns' rounding, 2^-62 of their largest entries: an FP64 sum rounds by 2^-53 of its
-// terms, and ran at the rate of the FP64 pipe: three products of 1,048,576 x 32 x 32 columns 6.5 ms, now 2.0.
+// terms, and ran at the rate of the FP64 pipe: three products of 1,048,576 x 32 x 32 columns 6.5 ms, now 2.2.
 template <typename S>
 tt_status xg_cross(cudaStream_t s, int num_sms, const XgPair<S>& pr, long nrows, Bump& ws, double* W, int* nonfinite,
                    int* status) {
@@ -1365,6 +1436,7 @@ tt_status xg_cross(cudaStream_t s, int num_sms, const XgPair<S>& pr, long nrows,
   unsigned char* da = ws.take<unsigned char>((size_t)aa.npiece * aa.po * aa.cpad * (NS * 16));
   unsigned char* db = nmat == 1 ? da : ws.take<unsigned char>((size_t)ab.npiece * ab.po * ab.cpad * (NS * 16));
   unsigned long long* gint = ws.take<unsigned long long>(3 * plane);
+  unsigned long long* cover = ws.take<unsigned long long>(plane);
   XgArgs args{};
   args.po = aa.po;
   args.parts = aa.parts;
@@ -1383,6 +1455,17 @@ tt_status xg_cross(cudaStream_t s, int num_sms, const XgPair<S>& pr, long nrows,
     const long grid = need < 8L * num_sms ? need : 8L * num_sms;
     k_xg_colmax<S><<<(unsigned)(grid > 0 ? grid : 1), 256, 0, s>>>(i ? pr.B : pr.A, ar.ncol, ar.sr, ar.sc, nrows,
                                                                    slots + (i ? pr.na : 0), nullptr, 0, ar.G, nonfinite);
+    count_launch();
+  }
+  {
+    const unsigned long long* sb = slots + (nmat == 1 ? 0 : pr.na);
+    const long stride = nrows / kXgCoverRows | 1, need = (nrows / stride + 64) / 64;
+    cudaMemsetAsync(cover, 0, 8 * plane, s);
+    k_xg_cover<S><<<dim3((unsigned)(need < 2L * num_sms ? need : 2L * num_sms), (unsigned)((pr.na + 15) / 16 * ((pr.nb + 15) / 16))),
+                    256, 0, s>>>(pr.A, pr.B, pr.na, pr.nb, nrows, stride, slots, sb, cover);
+    count_launch();
+    k_xg_cover_check<S><<<(unsigned)((plane + 255) / 256), 256, 0, s>>>(
+        pr.na, pr.nb, 1048576.0 / 512.0 * sqrt((double)nrows), slots, sb, cover, nonfinite);
     count_launch();
   }
   args.dig[0] = da;

@@ -44,6 +44,20 @@ def test_dot_keeps_what_is_not_finite(tt, value):
     assert np.isfinite(tt.tt_dot(tt.Context(0), y, y).item())
 
 
+@pytest.mark.parametrize("dtype,scale", [("f64", 1.0), ("f64", 1e-280), ("f32", 1.0), ("f32", 1e-30)])
+def test_dot_of_fields_that_are_large_on_different_rows(tt, dtype, scale):
+    # positive entries: an FP64 sum is within (rows + angles) 2^-53 = 1.9e-12 of the value, twice that for both sides
+    rng = np.random.default_rng(5)
+    rows, far = 16400, np.arange(16400) < 8200
+    a = [scale * rng.uniform(0.5, 1.0, (1, rows, 3)) * np.where(far, 1.0, 1e-12)[None, :, None], rng.uniform(0.5, 1.0, (3, 40, 1))]
+    b = [rng.uniform(0.5, 1.0, (1, rows, 2)) * np.where(far, 1e-12, 1.0)[None, :, None], rng.uniform(0.5, 1.0, (2, 40, 1))]
+    if dtype == "f32":
+        a, b = ([c.astype(np.float32).astype(np.float64) for c in t] for t in (a, b))
+    x, y = tt.TT.from_cores(a, rcap=[3], dtype=dtype), tt.TT.from_cores(b, rcap=[2], dtype=dtype)
+    want = float(np.sum((a[0][0].T @ b[0][0]) * (a[1][:, :, 0] @ b[1][:, :, 0].T)))
+    assert abs(tt.tt_dot(tt.Context(0), x, y).item() - want) <= 4e-12 * want
+
+
 WORKLOADS = [
     (plane_config1(nx=9, ny=7, G=5, ntheta=4, nphi=8, rmax=8).with_(
         inflow_temperature=(0.9, None, 0.6, None, None, 0.7)), 8, 48),
