@@ -13,6 +13,9 @@
 // the rotation's angle is formed in FP32 (the rotation itself is orthogonal to FP64 round-off; an angle
 // accurate to 2^-22 only costs a sweep's final factor).
 #pragma once
+#include <map>
+#include <mutex>
+
 #include "common.cuh"
 #include "instr.cuh"
 #include "xchol.cuh"
@@ -439,10 +442,17 @@ inline tt_status launch_jacobi_cl_e(cudaStream_t s, int n, int C, const double* 
   count_launch();
   return TT_OK;
 }
-// Whether clusters of 16 CTAs of the kernel can run (asked once per kernel).
+// Whether clusters of 16 CTAs of the kernel can run (asked once per kernel and context).
 template <typename T, int E>
 inline bool jc_wide_ok(int n) {
-  static const bool ok = [&] {
+  // per CUDA context: one that is destroyed and re-created needs the attribute again
+  static std::mutex mu;
+  static std::map<unsigned long long, bool> done;
+  const unsigned long long cid = current_context_id();
+  std::lock_guard<std::mutex> lock(mu);
+  const auto it = done.find(cid);
+  if (cid != 0 && it != done.end()) return it->second;
+  const bool ok = [&] {
     auto kern = k_jacobi_cl<T, E>;
     if (cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess) {
       (void)cudaGetLastError();
@@ -466,6 +476,7 @@ inline bool jc_wide_ok(int n) {
     return nc > 0;
   }();
   (void)n;
+  if (cid != 0) done[cid] = ok;
   return ok;
 }
 template <typename T, int E>
