@@ -60,9 +60,10 @@ def leaf_traffic(precision, variant, leaves, nrows):
     rd, wr, lm = t
     return rd * nrows / 589824 + wr * leaves / lm
 PREC_TEXT = {"fp64": "fp64",
-             "mixed": "mixed: f32 passes over the merged core (FP32 FMA), f64 small cores",
-             "mixed_3xtf32": "mixed_3xtf32: f32 passes over the merged core, the update GEMM on the tensor cores "
-                             "(tcgen05 kind::tf32, split 3xTF32 products, FP32 accumulation), f64 small cores"}
+             "mixed": "mixed: f32 passes over the merged core (exact digit products on the tensor cores, tcgen05 "
+                      "kind::f16), f64 small cores",
+             "mixed_3xtf32": "mixed_3xtf32: as mixed; updates of fewer rows than the digits take as split-TF32 products "
+                             "(tcgen05 kind::tf32, FP32 accumulation), f64 small cores"}
 
 
 def parse():
@@ -301,6 +302,8 @@ def time_precision(tt, torch, ctx, plan, wl, args, precision, dist, clocks_index
     stream = ctx.stream
     energy = torch.zeros(4, dtype=torch.float64, device="cuda")
     pinned = None
+    # what a choice equal to the default reports (the factor from exact Gram products)
+    default = ctx.get_tsqr(precision, (2 * wl.ndim + 1) * wl.rmax)
     if rounding == "tsqr" and args.tsqr:
         # pinned choice (e.g. the autotuner's, to profile the same kernels without timing
         # trials), in force from the first warm-up step on
@@ -391,38 +394,47 @@ def time_precision(tt, torch, ctx, plan, wl, args, precision, dist, clocks_index
     variant = tune["transport"][0] if tune is not None else "column"
     kname = {"column": "k_tsqr_leaf", "rowsplit": "k_tsqr_leaf_rs",
              "column_dense": "k_tsqr_leaf (32-row blocks, 4 CTAs/SM)"}[variant]
-    out["roofline"] = {"kernel": kname + " over the transport sum (one launch per step, R1 = 5r columns)",
-                       "bound": "alu", "achieved": leaf_tf, "peak": peak, "unit": "TFLOP/s",
-                       "frac": (leaf_tf / peak) if leaf_tf else None,
-                       "traffic": leaf_traffic(precision, variant, int(tune["transport"][1]) if tune else 0, wl.nrow),
-                       "traffic_note": ("ncu DRAM bytes (read + written) of this leaf kernel on the 96 x 96 workload, "
-                                        "reads scaled by rows and writes by leaves; null when no capture of the kernel "
-                                        "source as it stands is recorded"),
-                       "flops_per_launch": "2 N_Z R1^2 (R1 = 5 r, r the rank entering the step)",
-                       "peak_source": ("FP64" if precision == "fp64" else "FP32") + " FMA pipe, " + pk["source"] +
-                                      " in this run (tt_peak_probe)",
-                       "share": (kms["tsqr_leaf"] / nb) / (total_ms / args.steps) if total_ms else None}
-    # the first update pass (Z_new = Z_sum W over the transport sum, K = R1, N = r'): on the tensor
-    # cores in the 3xTF32 leg (three kind::tf32 MMAs per product), FP32 FMA otherwise
+    exact = rounding != "randomized" and (tune is None or (pinned is None and tuple(tune["transport"]) == tuple(default)))
+    ns = 8 if precision == "fp64" else 4  # digits of a column
+    # kind::f16 runs at twice the kind::tf32 rate
+    f16_peak = 2.0 * peaks["tf32_tensor"]["tflops"]
+    f16_source = "twice the kind::tf32 rate, " + peaks["tf32_tensor"]["source"] + " in this run (tt_peak_probe)"
+    if exact:
+        dig_tf = leaf_tf * ns * ns / 2.0 if leaf_tf else None
+        out["roofline"] = {"kernel": "k_xg_mma with its digits and sums over the transport sum (exact Gram products, "
+                                     "R1 = 5r columns)",
+                           "bound": "tensor", "achieved": dig_tf, "peak": f16_peak, "unit": "TFLOP/s",
+                           "frac": dig_tf / f16_peak if dig_tf else None, "algorithmic_tflops": leaf_tf, "traffic": None,
+                           "flops_per_launch": "%d N_Z R1^2 kind::f16 flops (%d digits a column, upper triangle; algorithmic "
+                                               "2 N_Z R1^2)" % (ns * ns, ns),
+                           "peak_source": f16_source,
+                           "share": (kms["tsqr_leaf"] / nb) / (total_ms / args.steps) if total_ms else None}
+    else:
+        out["roofline"] = {"kernel": kname + " over the transport sum (one launch per step, R1 = 5r columns)",
+                           "bound": "alu", "achieved": leaf_tf, "peak": peak, "unit": "TFLOP/s",
+                           "frac": (leaf_tf / peak) if leaf_tf else None,
+                           "traffic": leaf_traffic(precision, variant, int(tune["transport"][1]) if tune else 0, wl.nrow),
+                           "traffic_note": ("ncu DRAM bytes (read + written) of this leaf kernel on the 96 x 96 workload, "
+                                            "reads scaled by rows and writes by leaves; null when no capture of the kernel "
+                                            "source as it stands is recorded"),
+                           "flops_per_launch": "2 N_Z R1^2 (R1 = 5 r, r the rank entering the step)",
+                           "peak_source": ("FP64" if precision == "fp64" else "FP32") + " FMA pipe, " + pk["source"] +
+                                          " in this run (tt_peak_probe)",
+                           "share": (kms["tsqr_leaf"] / nb) / (total_ms / args.steps) if total_ms else None}
+    # the first update pass (Z_new = Z_sum W over the transport sum, K = R1, N = r'): from digits on the
+    # tensor cores (products of digits i + j below the orders kept: 13 for FP32 passes, 36 for FP64)
     up_flops = 0.0
     for i in range(nb):
         up_flops += 2.0 * N * (5 * b_ranks[i][1]) * b_ranks[i + 1][1]
     if kms["update"] > 0:
         up_alg = up_flops / (kms["update"] / 1e3) / 1e12
-        if precision == "mixed_3xtf32":
-            tp = peaks["tf32_tensor"]
-            out["roofline_update"] = {
-                "kernel": "k_update_tc (tcgen05 kind::tf32, 3xTF32, 128-row tiles, one CTA per SM)",
-                "bound": "tensor", "achieved": 3.0 * up_alg, "peak": tp["tflops"], "unit": "TFLOP/s",
-                "frac": 3.0 * up_alg / tp["tflops"], "algorithmic_tflops": up_alg,
-                "flops_per_launch": "3 x 2 N_Z R1 r' tensor-pipe flops (three TF32 products per FP32 product)",
-                "peak_source": "kind::tf32 tensor pipe, " + tp["source"] + " in this run (tt_peak_probe)",
-                "ms_per_launch": kms["update"] / nb}
-        else:
-            out["roofline_update"] = {
-                "kernel": ("k_update (FP64)" if precision == "fp64" else "k_update_blk (FP32 FMA)"),
-                "bound": "alu", "achieved": up_alg, "peak": peak, "unit": "TFLOP/s", "frac": up_alg / peak,
-                "flops_per_launch": "2 N_Z R1 r'", "ms_per_launch": kms["update"] / nb}
+        pairs = 36 if precision == "fp64" else 13
+        out["roofline_update"] = {
+            "kernel": "k_update_dig (tcgen05 kind::f16, base-256 digits) with its row and weight scales",
+            "bound": "tensor", "achieved": pairs * up_alg, "peak": f16_peak, "unit": "TFLOP/s",
+            "frac": pairs * up_alg / f16_peak, "algorithmic_tflops": up_alg,
+            "flops_per_launch": "%d x 2 N_Z R1 r' kind::f16 flops (digit products kept)" % pairs,
+            "peak_source": f16_source, "ms_per_launch": kms["update"] / nb}
     ctx.set_rounding("tsqr")
     return out, x, energy
 
@@ -497,16 +509,7 @@ def run_ours(args):
         G = results["fp64_gram"]
         line["fp64_gram"] = {k: G[k] for k in ("value", "ms_per_step", "tflops", "breakdown_ms_per_step",
                                                "gpu_launches", "ranks", "jacobi")}
-        # the Gram pass over the transport sum (symmetric: N R1 (R1 + 1) flops at R1 = 5r)
-        rh = G["rank_history"]
-        gflops = sum(2.0 * wl.nrow * (5 * r[0]) * (5 * r[0] + 1) / 2.0 for r in rh[:-1])
-        gms = G["breakdown_ms_per_step"]["tsqr_leaf"] * args.steps
-        ach = gflops / (gms / 1e3) / 1e12 if gms > 0 else None
-        line["fp64_gram"]["roofline"] = {
-            "kernel": "k_gram_tiles + k_gram_reduce over the transport sum (FP64 Gram, upper triangle)",
-            "bound": "alu", "achieved": ach, "peak": peaks["fp64"]["tflops"], "unit": "TFLOP/s",
-            "frac": ach / peaks["fp64"]["tflops"] if ach else None,
-            "peak_source": "FP64 FMA pipe, " + peaks["fp64"]["source"] + " in this run (tt_peak_probe)"}
+        line["fp64_gram"]["roofline"] = G["roofline"]
         Eg = tt.tt_energy_density(ctx, plan, states["fp64_gram"]).cpu().numpy()
         Ed = tt.tt_energy_density(ctx, plan, states["fp64"]).cpu().numpy()
         line["fp64_gram"]["energy_density_rel_err_vs_tsqr"] = float(np.linalg.norm(Eg - Ed) / np.linalg.norm(Ed))
