@@ -30,7 +30,7 @@ __device__ __forceinline__ double tr_scaled(double lam, float, float, double a, 
 // Merged core of the materialised transport sum in compact layout: columns t*r + q
 // (t = 0 state, t = 1..nterm operator images) and the nbc inflow columns after them.  A thread keeps
 // one column (its operator is looked up once), a CTA takes 64 rows at a time (their neighbour flags are
-// formed once, by 64 threads), four rows of a thread in flight.  1,048,576 x 160 FP32: 0.43 ms (671 MB written); with a
+// formed once, by 64 threads), four rows of a thread in flight.  1,048,576 x 81 FP32: 0.37 ms (340 MB written); with a
 // thread per entry, which divided for its row, column and neighbours in 64 bits and scaled in FP64: 1.47 ms.
 constexpr int kTrRows = 64;
 // SrcStencil::row_flags in 32 bits where the rows allow it (64-bit division runs on the FP64 pipe).
