@@ -99,10 +99,11 @@ tt_status same_modes(const tt_tensor* a, const tt_tensor* b);
 
 // Unique id of the CUDA context current on the calling thread (0 when none is current).
 unsigned long long current_context_id();
-// Allow `bytes` of dynamic shared memory per CTA for kernel `func` (the opt-in above 48 KB),
-// never lowering an earlier setting.  TT_ERR_CUDA if the runtime refuses, TT_ERR_UNSUPPORTED
-// above the device's opt-in maximum.  Every launch site above 48 KB calls it and returns its
-// status, so a refused attribute never reaches a launch (or a captured graph node).
+// Allow `bytes` of dynamic shared memory per CTA for kernel `func` (the opt-in above 48 KB, the kernel's
+// static arrays included), never lowering an earlier setting.  TT_ERR_CUDA if the runtime refuses,
+// TT_ERR_UNSUPPORTED above the device's opt-in maximum.  Every launch site that may take more than 48 KB
+// with its static arrays calls it and returns its status, so a refused attribute never reaches a launch
+// (or a captured graph node).
 tt_status smem_optin_impl(const void* func, size_t bytes);
 template <class F>
 inline tt_status smem_optin(F* func, size_t bytes) {

@@ -1,5 +1,5 @@
 // Host runtime helpers shared by every translation unit: the identity of the current CUDA
-// context and the checked opt-in to more than 48 KB of dynamic shared memory per CTA.
+// context and the checked opt-in to more than 48 KB of shared memory per CTA.
 #include <map>
 #include <mutex>
 #include <utility>
@@ -40,9 +40,10 @@ unsigned long long current_context_id() {
 }
 
 // Largest dynamic shared memory already allowed, per (kernel, context).  A context that is
-// destroyed and re-created (cudaDeviceReset) gets a new id, so its kernels are set again.
+// destroyed and re-created (cudaDeviceReset) gets a new id, so its kernels are set again.  Without the
+// opt-in a CTA gets 48 KB in all: a kernel's static arrays count, so the limit is the kernel's own.
 tt_status smem_optin_impl(const void* func, size_t bytes) {
-  if (bytes <= 48 * 1024) return TT_OK;
+  if (bytes == 0) return TT_OK;
   static std::mutex mu;
   static std::map<std::pair<const void*, unsigned long long>, size_t> done;
   const unsigned long long cid = current_context_id();
@@ -58,13 +59,13 @@ tt_status smem_optin_impl(const void* func, size_t bytes) {
     (void)cudaGetLastError();
     return TT_ERR_CUDA;
   }
-  if (bytes > (size_t)optin) return TT_ERR_UNSUPPORTED;
-  // never lower a limit that an earlier launch (or a captured graph node) relies on
   cudaFuncAttributes fa;
   if (cudaFuncGetAttributes(&fa, func) != cudaSuccess) {
     (void)cudaGetLastError();
     return TT_ERR_CUDA;
   }
+  if (bytes + fa.sharedSizeBytes > (size_t)optin) return TT_ERR_UNSUPPORTED;
+  // never lower a limit that an earlier launch (or a captured graph node) relies on
   if ((size_t)fa.maxDynamicSharedSizeBytes < bytes &&
       cudaFuncSetAttribute(func, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes) != cudaSuccess) {
     (void)cudaGetLastError();
