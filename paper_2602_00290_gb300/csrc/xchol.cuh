@@ -12,7 +12,8 @@
 // the integer rate, and a double-double update (20 FP64 operations) would take 4 ms at 160 columns.
 //
 // Right-looking, one cluster: CTA r holds the columns i = r mod C (all rows), the pivot's row is
-// exchanged through distributed shared memory, one cluster barrier per step.  Every CTA keeps all
+// exchanged through distributed shared memory, one cluster barrier per step (and one before the first
+// exchange: a peer's shared memory may be written only once that CTA runs).  Every CTA keeps all
 // diagonals (r_p is known to all of them), so pivots and reciprocal square roots need no exchange; the
 // next pivot's row is updated and sent first, the rest of the update and the next reciprocal square
 // root run between the barrier's arrival and its wait.
@@ -156,6 +157,7 @@ __global__ void __launch_bounds__(kXcThreads) k_xg_chol(int n, const unsigned lo
   __shared__ __align__(16) unsigned wkey[2][kXcMaxN / 32];
   const int C = (int)xc_cluster_size(), rank = (int)xc_cluster_rank();
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  if (C > 1) xc_arrive();  // this CTA runs (waited for before the first exchange)
   const int ncl = xc_cols(n, C);
   const size_t plane = (size_t)n * n;
   SI* S = reinterpret_cast<SI*>(xc_smem);  // [ncl][n]: column lc C + rank; row of a finished pivot: r
@@ -247,6 +249,7 @@ __global__ void __launch_bounds__(kXcThreads) k_xg_chol(int n, const unsigned lo
   // threads of the row exchange: one per (own column, destination)
   const int xl = tid / C, xd = tid - (tid / C) * C, xi = xl * C + rank;
   const bool xon = xl < ncl && xi < na;
+  if (C > 1) xc_wait();  // every CTA of the cluster runs
   if (key) {
     if (xon) send(rowbuf + xi, xd, S[(size_t)xl * n + pv]);
     arrive();
