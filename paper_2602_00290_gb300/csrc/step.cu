@@ -355,6 +355,15 @@ inline int xg_sms(const tt_context* ctx) {
   return share < ctx->num_sms ? share : ctx->num_sms;
 }
 
+// Whether the factor of the rounding gives the digit update its column sizes (else the columns do).
+inline bool ud_scales_from_factor(const tt_context* ctx) { return ctx->rounding == TT_ROUND_TSQR; }
+template <class Src>
+inline tt_status ud_scales(const tt_context* ctx, cudaStream_t s, const Src& src, const LivePattern& lp, long nrows,
+                           const double* RZ, const UdBufs& ub) {
+  if (ud_scales_from_factor(ctx)) return launch_ud_scales(s, RZ, lp.ncap(), ub);
+  return launch_ud_scales_cols(s, ctx->num_sms, src, lp, nrows, ub);
+}
+
 // Whether a pass's update runs from digits on the tensor cores (update_dig.cuh), and its buffers.
 template <typename T, class Src>
 inline bool take_ud(const tt_context* ctx, const Src& src, const LivePattern& lp, long nrows, int kcap, Bump& ws,
@@ -363,7 +372,9 @@ inline bool take_ud(const tt_context* ctx, const Src& src, const LivePattern& lp
   if constexpr (sizeof(T) == 4 && std::is_same<Src, SrcStencil<float>>::value) {
     if (ctx->tensor_cores && nrows < kUdMinRowsTc && update_tc_fits(src, lp, nrows, kcap, ctx->smem_optin)) return false;
   }
+  if (!ud_scales_from_factor(ctx) && ud_storage_cols(src, lp) > 256) return false;
   ub.cexp = ws.take<int>(lp.ncap());
+  if (!ud_scales_from_factor(ctx)) ub.slots = ws.take<unsigned long long>(ud_storage_cols(src, lp) + lp.nextra);
   if (XgElem<Src>::stencil) ub.rho = ws.take<short>(nrows);
   ub.w = ws.take<unsigned char>(update_dig_wbytes<T>(src, lp, kcap));
   int* rinfo = ws.take<int>(nrows);
@@ -520,7 +531,7 @@ tt_status round_impl(tt_context* ctx, tt_tensor* x, double tol, int rmax, Bump& 
   job.RZ = RZ;
   UdBufs ub;
   tt_status st = TT_OK;
-  if (take_ud<T>(ctx, src, lp, N, K1, ws, ub)) st = launch_ud_scales(s, RZ, R, ub);
+  if (take_ud<T>(ctx, src, lp, N, K1, ws, ub)) st = ud_scales(ctx, s, src, lp, N, RZ, ub);
   if (st == TT_OK) st = small_round(s, ctx->num_sms, job, ws);
   if (st != TT_OK || ws.dry) return st;
   st = launch_update<T>(ctx, s, ctx->num_sms, SrcRows<S>{(const S*)x->core[0], K1}, lp, N, b.W, K1,
@@ -619,7 +630,7 @@ tt_status step_impl(tt_context* ctx, const tt_plan* p, tt_tensor* I, double tol,
   j1.RZ = RZ1;
   UdBufs ub1, ub2;
   tt_status st = TT_OK;
-  if (take_ud<T>(ctx, src1, lp1, N, K1, ws, ub1)) st = launch_ud_scales(s, RZ1, R1, ub1);
+  if (take_ud<T>(ctx, src1, lp1, N, K1, ws, ub1)) st = ud_scales(ctx, s, src1, lp1, N, RZ1, ub1);
   if (st == TT_OK) st = small_round(s, ctx->num_sms, j1, ws);
   if (st != TT_OK) return st;
   // ---- source step fused into the write of the rounded transport update
@@ -697,7 +708,7 @@ tt_status step_impl(tt_context* ctx, const tt_plan* p, tt_tensor* I, double tol,
   j2.core2 = b2.core2;
   j2.Bnew = b2.Bnew;
   j2.vJ = b2.vJ;
-  if (ud2) st = launch_ud_scales(s, RZ2, lp2.ncap(), ub2);
+  if (ud2) st = ud_scales(ctx, s, SrcRows<S>{Zsrc, K1 + 1}, lp2, N, RZ2, ub2);
   if (st == TT_OK) st = small_round(s, ctx->num_sms, j2, ws);
   if (st != TT_OK) return st;
   st = launch_update<T>(ctx, s, ctx->num_sms, SrcRows<S>{Zsrc, K1 + 1}, lp2, N, b2.W, K1,

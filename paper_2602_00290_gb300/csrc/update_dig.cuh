@@ -45,7 +45,8 @@ constexpr int kUdMinExp = -8000;                 // row scale of a zero row
 
 // Scales of a pass and where its weights' digits go (workspace).
 struct UdBufs {
-  int* cexp = nullptr;        // [ncap] size of each column: exponent of its largest entry in RZ
+  int* cexp = nullptr;        // [ncap] size of each column (launch_ud_scales, launch_ud_scales_cols)
+  unsigned long long* slots = nullptr;  // [columns] largest entries (launch_ud_scales_cols)
   short* rho = nullptr;       // [nrows] exponent of a storage row (stencil passes)
   int* rinfo = nullptr;       // [nrows] scale of a row of the pass (16 bits), neighbour flags from bit 16
   unsigned char* w = nullptr; // digits of the weights, exponents
@@ -141,6 +142,17 @@ __global__ void __launch_bounds__(128) k_ud_colexp(const double* __restrict__ RZ
   if ((threadIdx.x & 31) == 0) atomicMax(&m, e);
   __syncthreads();
   if (threadIdx.x == 0) cexp[c] = m ? m - 1023 : 0;
+}
+
+// Exponent of every storage column's largest entry (slots, k_xg_colmax) and, behind the operators' columns, of the
+// inflow columns'; the operators' own columns have no digits of their own.
+static __global__ void __launch_bounds__(256) k_ud_slotexp(int ncol, int extra0, int nextra,
+                                                    const unsigned long long* __restrict__ slots,
+                                                    int* __restrict__ cexp) {
+  for (int c = threadIdx.x; c < ncol + nextra; c += blockDim.x) {
+    const int e = (int)((slots[c] >> 52) & 0x7ff);
+    cexp[c < ncol ? c : extra0 + c - ncol] = e ? e - 1023 : 0;
+  }
 }
 
 __device__ __forceinline__ int ud_exp(double x) { return (int)((__double_as_longlong(x) >> 52) & 0x7ff) - 1023; }
@@ -850,10 +862,50 @@ inline size_t update_dig_wbytes(const Src& src, const LivePattern& lp, int kcap)
   return ud_b_bytes(nunit, NS, kp) + sizeof(int) * (size_t)(kp + 16 * nunit);
 }
 
-// The scales need RZ (the triangular factor of the pass's columns, ncap x ncap row-major) before it is
-// overwritten: called first, then launch_update_dig.
+// Columns of the storage matrix of a pass, and where its inflow columns stand.
+template <typename S>
+inline int ud_storage_cols(const SrcStencil<S>& s, const LivePattern&) { return s.rcap; }
+template <typename S>
+inline int ud_storage_cols(const SrcRows<S>&, const LivePattern& lp) { return lp.ncap(); }
+
+// Column sizes, called before launch_update_dig.  From RZ (ncap x ncap row-major, before it is overwritten) where
+// it is the triangular factor of the pass's columns to their own accuracy (R^T R = A^T A column by column):
 inline tt_status launch_ud_scales(cudaStream_t s, const double* RZ, int n, const UdBufs& ub) {
   k_ud_colexp<<<(unsigned)n, 128, 0, s>>>(RZ, n, ub.cexp);
+  count_launch();
+  return cudaGetLastError() == cudaSuccess ? TT_OK : TT_ERR_CUDA;
+}
+
+// From the columns themselves where it is not: a Gram matrix's factor ends at pivots of 4 n eps of its largest
+// diagonal entry and a sketch's keeps the columns' parts in its range, so a column may be far larger than RZ says; a
+// row's scale follows that column, and the other columns of the row lost as many bits (nine orthogonal columns
+// graded 1 to 1e-12: the state to 1 %).  One more pass over the storage (1,048,576 x 32 FP64: 0.05 ms).
+template <class Src>
+tt_status launch_ud_scales_cols(cudaStream_t s, int num_sms, const Src& src, const LivePattern& lp, long nrows,
+                                const UdBufs& ub) {
+  using S = typename XgElem<Src>::type;
+  const int ncol = ud_storage_cols(src, lp);
+  int nextra = 0, extra0 = 0, G = 1;
+  const double* bc = nullptr;
+  const S* A = nullptr;
+  long ld = 0;
+  if constexpr (XgElem<Src>::stencil) {
+    nextra = lp.nextra;
+    extra0 = (src.nterm + 1) * src.rcap;
+    G = src.G;
+    bc = src.bcval;
+    A = src.Z;
+    ld = src.ldz;
+  } else {
+    A = src.A;
+    ld = src.ld;
+  }
+  if (cudaMemsetAsync(ub.slots, 0, sizeof(unsigned long long) * (size_t)(ncol + nextra), s) != cudaSuccess)
+    return TT_ERR_CUDA;
+  k_xg_colmax<S><<<xg_colmax_grid(num_sms, ncol, nrows), 256, 0, s>>>(A, ncol, ld, 1, nrows, ub.slots, bc, nextra, G,
+                                                                      nullptr);
+  count_launch();
+  k_ud_slotexp<<<1, 256, 0, s>>>(ncol, extra0, nextra, ub.slots, ub.cexp);
   count_launch();
   return cudaGetLastError() == cudaSuccess ? TT_OK : TT_ERR_CUDA;
 }

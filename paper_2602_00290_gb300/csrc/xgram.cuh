@@ -1167,17 +1167,21 @@ tt_status xg_launch_products(cudaStream_t s, const XgPlan& pl, XgArgs& args, lon
   count_launch();
   return cudaGetLastError() == cudaSuccess ? TT_OK : TT_ERR_CUDA;
 }
+// CTAs of k_xg_colmax over nrows rows of ncol <= 256 columns.
+inline unsigned xg_colmax_grid(int num_sms, int ncol, long nrows) {
+  const long rpb = 256 / ncol, need = (nrows + 8 * rpb - 1) / (8 * rpb);
+  const long grid = need < 8L * num_sms ? need : 8L * num_sms;
+  return (unsigned)(grid > 0 ? grid : 1);
+}
 template <int NS, typename S>
 void xg_launch_digits(cudaStream_t s, int num_sms, const S* A, const XgArray& ar, LivePattern lp, long nrows,
                       unsigned long long* slots, unsigned char* dig, const double* bc, int nbc, unsigned char* bcdig,
                       int* nonfinite = nullptr) {
-  const long rpb = 256 / ar.ncol, need = (nrows + 8 * rpb - 1) / (8 * rpb);
-  long grid = need < 8L * num_sms ? need : 8L * num_sms;
-  k_xg_colmax<S><<<(unsigned)(grid > 0 ? grid : 1), 256, 0, s>>>(A, ar.ncol, ar.sr, ar.sc, nrows, slots, bc, nbc, ar.G,
-                                                                     nonfinite);
+  k_xg_colmax<S><<<xg_colmax_grid(num_sms, ar.ncol, nrows), 256, 0, s>>>(A, ar.ncol, ar.sr, ar.sc, nrows, slots, bc, nbc,
+                                                                         ar.G, nonfinite);
   count_launch();
   const long tot = ar.npiece * ar.po * ar.cpad;
-  grid = (tot + 255) / 256;
+  long grid = (tot + 255) / 256;
   if (grid > 16L * num_sms) grid = 16L * num_sms;
   k_xg_digits<NS, S><<<(unsigned)(grid > 0 ? grid : 1), 256, 0, s>>>(A, ar, lp, nrows, slots, dig, bc, nbc, bcdig);
   count_launch();
@@ -1451,10 +1455,9 @@ tt_status xg_cross(cudaStream_t s, int num_sms, const XgPair<S>& pr, long nrows,
   cudaMemsetAsync(nonfinite, 0, sizeof(int), s);
   for (int i = 0; i < nmat; ++i) {
     const XgArray& ar = i ? ab : aa;
-    const long rpb = 256 / ar.ncol, need = (nrows + 8 * rpb - 1) / (8 * rpb);
-    const long grid = need < 8L * num_sms ? need : 8L * num_sms;
-    k_xg_colmax<S><<<(unsigned)(grid > 0 ? grid : 1), 256, 0, s>>>(i ? pr.B : pr.A, ar.ncol, ar.sr, ar.sc, nrows,
-                                                                   slots + (i ? pr.na : 0), nullptr, 0, ar.G, nonfinite);
+    k_xg_colmax<S><<<xg_colmax_grid(num_sms, ar.ncol, nrows), 256, 0, s>>>(i ? pr.B : pr.A, ar.ncol, ar.sr, ar.sc, nrows,
+                                                                           slots + (i ? pr.na : 0), nullptr, 0, ar.G,
+                                                                           nonfinite);
     count_launch();
   }
   {
