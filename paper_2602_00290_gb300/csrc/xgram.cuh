@@ -1324,15 +1324,16 @@ struct XgPair {
 };
 template <typename S>
 struct XgElem<XgPair<S>> { using type = S; static constexpr bool stencil = false; };
+constexpr int kXgPairCols = 256;  // columns of either matrix
 template <int NS, typename S>
 inline bool xg_make_plan(const XgPair<S>& s, const LivePattern&, XgPlan& pl) {
   pl.nsub = 0;
   pl.nraw = s.na + s.nb;
-  return s.na <= 256 && s.nb <= 256 && xg_add<NS>(pl, s.na, 0, 0, 0) && xg_add<NS>(pl, s.nb, s.na, 1, 0) &&
+  return s.na <= kXgPairCols && s.nb <= kXgPairCols && xg_add<NS>(pl, s.na, 0, 0, 0) && xg_add<NS>(pl, s.nb, s.na, 1, 0) &&
          xg_tiles<NS>(pl, true) && xg_stages(pl) >= 2;
 }
 template <typename S>
-inline long xg_plan_key(const XgPair<S>& s, const LivePattern&) { return 1000L * s.na + s.nb; }
+inline long xg_plan_key(const XgPair<S>& s, const LivePattern&) { return ((long)s.na << 32) | (long)s.nb; }
 
 // Whether the fixed point holds an inner product as well as FP64 sums do.  A column's rounding is 2^-62 of its
 // largest entry, so a product of N rows is off by about 2^-62 sqrt(N) max|a| max|b|, an FP64 sum by 2^-53 of
@@ -1408,6 +1409,7 @@ __global__ void __launch_bounds__(256) k_xg_cover_check(int na, int nb, double l
 constexpr long kXgCrossRows = 1L << 18;
 template <typename S>
 inline const XgPlan* xg_cross_plan(const XgPair<S>& pr) {
+  if (pr.na > kXgPairCols || pr.nb > kXgPairCols) return nullptr;
   // a matrix with itself: the upper triangle
   if (pr.A == pr.B && pr.na == pr.nb) return xg_plan_of<8>(SrcRows<S>{pr.A, pr.na}, LivePattern{nullptr, pr.na, 1, 0});
   return xg_plan_of<8>(pr, LivePattern{nullptr, 1, 1, 0});
