@@ -517,17 +517,32 @@ inline bool ud_vec(const SrcStencil<S>& s) {
 template <typename S>
 inline bool ud_vec(const SrcRows<S>& s) { return ((size_t)s.ld * sizeof(S)) % 16 == 0 && (size_t)s.A % 16 == 0; }
 
-// s 2^e, rounded once (FP64, on the integer units: the FP64 pipe is narrow).
-__device__ __forceinline__ double ud_make(long long s, int e) {
-  if (s == 0) return 0.0;
-  const unsigned long long a = s < 0 ? 0ull - (unsigned long long)s : (unsigned long long)s;
-  const int lz = __clzll((long long)a);
-  const unsigned long long nm = a << lz;
-  const int f = 1023 + 63 - lz + e;
-  if (f < 2 || f > 2044) return ldexp((double)s, e);
+// (hi 2^32 + lo) 2^e, rounded once (FP64, on the integer units: the FP64 pipe is narrow).
+__device__ __forceinline__ double ud_make(long long hi, unsigned lo, int e) {
+  const bool neg = hi < 0;
+  if (neg) {
+    lo = 0u - lo;
+    hi = ~hi + (lo == 0u ? 1 : 0);
+  }
+  const unsigned long long a = (unsigned long long)hi, b = (unsigned long long)lo << 32;
+  int lz;
+  unsigned long long nm;  // the leading 64 bits
+  if (a != 0ull) {
+    lz = __clzll((long long)a);
+    nm = lz ? (a << lz) | (b >> (64 - lz)) : a;
+  } else {
+    if (lo == 0u) return 0.0;
+    lz = 64 + __clz((int)lo);
+    nm = b << (lz - 64);
+  }
+  const int f = 1023 + 95 - lz + e;
+  if (f < 2 || f > 2044) {
+    const double v = ldexp(__ull2double_rn(nm), f - 1086);
+    return neg ? -v : v;
+  }
   const unsigned long long m = (nm >> 11) + ((nm >> 10) & 1ull);
-  const unsigned long long b = ((unsigned long long)(f - 1) << 52) + m;
-  return __longlong_as_double((long long)(b | ((unsigned long long)s & 0x8000000000000000ull)));
+  const unsigned long long r = ((unsigned long long)(f - 1) << 52) + m;
+  return __longlong_as_double((long long)(r | (neg ? 0x8000000000000000ull : 0ull)));
 }
 
 template <int Q>
@@ -669,7 +684,9 @@ __global__ void __launch_bounds__(ud_threads(NS), 1)
               hi += (long long)__float2int_rn(__uint_as_float(v[o][b])) << (8 * (3 - o));
               lo += (long long)__float2int_rn(__uint_as_float(v[4 + o][b])) << (8 * (3 - o));
             }
-            val = ud_make(hi * 16384 + ((lo + 131072) >> 18), r + we[n0 + b] - 48);
+            // hi 2^32 + lo, every bit of it: cut to 64 bits (a unit of 2^-47 to 2^-50 of the row's largest
+            // possible product) outputs of nine columns were off by 6 to 16 times an FP64 sum's error
+            val = ud_make(hi + (lo >> 32), (unsigned)lo, r + we[n0 + b] - 66);
           }
           if constexpr (Epi::kDot) js[b & 3] = fma(val, vJs[n0 + b], js[b & 3]);
           O[(size_t)lane * (kp + 1) + n0 + b] = val;
