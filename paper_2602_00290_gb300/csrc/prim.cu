@@ -341,7 +341,21 @@ tt_status axpy_impl(tt_context* ctx, double alpha, const tt_tensor* x, tt_tensor
   return cudaGetLastError() == cudaSuccess ? TT_OK : TT_ERR_CUDA;
 }
 
+// Whether the first cores' products are formed exactly (xg_cross): the digits cost by rows and columns, the FP64 sums
+// by rows and products in groups of 256.  Inner products, exact / sums, cold L2, us:
+//   8,192 rows (the sums stay): 32 x 32 FP64 117 / 501, FP32 113 / 349; 1 x 1: 105 / 128, 104 / 169
+//   262,144 rows: 2 x 2 FP64 163 / 217, FP32 160 / 206; 32 x 32: 289 / 555, 275 / 1,523; 1 x 200 FP64 579 / 469
+//   1,048,576 rows: FP64 1 x 1 436 / 205, 8 x 8 472 / 477, 14 x 14 600 / 582, 16 x 16 603 / 639, 32 x 32 894 / 2,217;
+//     FP32 4 x 4 443 / 323, 6 x 6 451 / 496, 2 x 32 610 / 494, 8 x 8 460 / 506, 32 x 32 843 / 5,690
+// (a pass is 262,144 rows: beyond one, the exact form needs many products for each column whose digits it forms.)
 constexpr long kDotExactRows = 16384;
+template <typename S>
+inline bool dot_exact(const XgPair<S>& pr, long N) {
+  if (N < kDotExactRows || !xg_cross_fits(pr)) return false;
+  const long cols = xg_cross_same(pr) ? pr.na : pr.na + pr.nb, ne = (long)pr.na * pr.nb;
+  if (N <= kXgCrossRows && N * cols <= (1L << 25)) return true;
+  return ne >= (sizeof(S) == 8 ? 8 * cols : 3L * (pr.na + pr.nb));
+}
 template <typename S>
 tt_status dot_impl(tt_context* ctx, const tt_tensor* x, const tt_tensor* y, double* out, Bump& ws) {
   cudaStream_t s = ctx->stream;
@@ -359,11 +373,11 @@ tt_status dot_impl(tt_context* ctx, const tt_tensor* x, const tt_tensor* y, doub
   double* Bx = ws.take<double>((size_t)rx * nang);
   double* By = ws.take<double>((size_t)ry * nang);
   double* G = ws.take<double>(ne);
-  // tall cores: exact products on the tensor cores, the FP64 sums only where an entry is not finite or the columns
-  // are large on different rows (k_xg_cover).  From 16,384 rows on; fewer are a few microseconds either way
+  // tall cores: exact products on the tensor cores (dot_exact), the FP64 sums only where an entry is not finite or
+  // the columns are large on different rows (k_xg_cover)
   const XgPair<S> pr{(const S*)x->core[0], (const S*)y->core[0], rx, ry};
   int* when = nullptr;
-  if (!ctx->no_xg && N >= kDotExactRows && xg_cross_fits(pr)) {
+  if (!ctx->no_xg && dot_exact(pr, N)) {
     when = ws.take<int>(1);
     const tt_status st = xg_cross<S>(s, ctx->num_sms, pr, N, ws, W1, when, &ctx->ctrl->status);
     if (st != TT_OK) return st;

@@ -1408,10 +1408,12 @@ __global__ void __launch_bounds__(256) k_xg_cover_check(int na, int nb, double l
 // 65,536 rows a pass spent half of the time in k_xg_sum.
 constexpr long kXgCrossRows = 1L << 18;
 template <typename S>
+inline bool xg_cross_same(const XgPair<S>& pr) { return pr.A == pr.B && pr.na == pr.nb; }
+template <typename S>
 inline const XgPlan* xg_cross_plan(const XgPair<S>& pr) {
   if (pr.na > kXgPairCols || pr.nb > kXgPairCols) return nullptr;
   // a matrix with itself: the upper triangle
-  if (pr.A == pr.B && pr.na == pr.nb) return xg_plan_of<8>(SrcRows<S>{pr.A, pr.na}, LivePattern{nullptr, pr.na, 1, 0});
+  if (xg_cross_same(pr)) return xg_plan_of<8>(SrcRows<S>{pr.A, pr.na}, LivePattern{nullptr, pr.na, 1, 0});
   return xg_plan_of<8>(pr, LivePattern{nullptr, 1, 1, 0});
 }
 template <typename S>
@@ -1428,7 +1430,7 @@ tt_status xg_cross(cudaStream_t s, int num_sms, const XgPair<S>& pr, long nrows,
   constexpr int NS = 8, H = XgCfg<NS>::H, Wd = XgCfg<NS>::W;
   const LivePattern la{nullptr, pr.na, 1, 0}, lb{nullptr, pr.nb, 1, 0};
   const XgPlan& pl = *xg_cross_plan(pr);
-  const int nmat = pr.A == pr.B && pr.na == pr.nb ? 1 : 2;
+  const int nmat = xg_cross_same(pr) ? 1 : 2;
   const long rows = nrows < kXgCrossRows ? nrows : kXgCrossRows;
   XgArray aa, ab;
   const S* p = nullptr;

@@ -41,3 +41,21 @@ def test_dots_in_turn(tt, pairs, rows, dtype):
         for u, v, p, q in ((x, y, a, b), (y, x, b, a), (x, x, a, a)):
             norms = (inner(p, p) * inner(q, q)) ** 0.5
             assert abs(tt.tt_dot(ctx, u, v).item() - inner(p, q)) <= 1e-12 * norms
+
+
+def launches(tt, rows, rx, ry, dtype):
+    x, y = (tt.TT.from_cores(random_tt([rows, 8], [r], seed=r), dtype=dtype) for r in (rx, ry))
+    ctx = tt.Context(0)
+    ctx.counters(reset=True)
+    tt.tt_dot(ctx, x, y)
+    return sum(ctx.counters()[1].values())
+
+
+@pytest.mark.parametrize("rows,rx,ry,dtype,exact", [
+    (1000, 32, 32, "f64", False), (16384, 2, 3, "f64", True), (1 << 18, 2, 3, "f64", True), (1 << 18, 1, 140, "f64", False),
+    ((1 << 18) + 1, 2, 3, "f64", False), ((1 << 18) + 1, 15, 15, "f64", False), ((1 << 18) + 1, 16, 16, "f64", True),
+    ((1 << 18) + 1, 5, 5, "f32", False), ((1 << 18) + 1, 6, 6, "f32", True), ((1 << 18) + 1, 2, 32, "f32", False),
+])
+def test_narrow_products_of_many_rows_take_the_sums(tt, rows, rx, ry, dtype, exact):
+    # the exact form is several launches more; where it took longer than the sums, the sums stay
+    assert (launches(tt, rows, rx, ry, dtype) > launches(tt, 1000, rx, ry, dtype)) == exact
