@@ -151,7 +151,12 @@ const char *tt_status_string(tt_status s);
 /* Create a context bound to CUDA device `device` and stream `cuda_stream` (a cudaStream_t,
  * NULL = legacy default stream).  `workspace_bytes` > 0 pre-allocates that much device
  * workspace; 0 lets the library size it on first use (outside any stream capture).
- * The context owns its workspace and its device status word. */
+ * A call that needs more replaces it by a larger one after the stream's work (never under capture).  A
+ * workspace that a call used while the stream was being captured by the caller stays allocated until
+ * tt_context_destroy, so that the caller's graph may be replayed whatever the context does meanwhile.
+ * Where the larger workspace of the exact products (TT_ROUND_TSQR, tt_dot) cannot be had, the calls take
+ * the kernels that need less, and the context does not ask for that size again.
+ * The context owns its workspaces and its device status word. */
 tt_status tt_context_create(tt_context **ctx, int device, void *cuda_stream, size_t workspace_bytes);
 tt_status tt_context_destroy(tt_context *ctx);
 
@@ -283,7 +288,8 @@ tt_status tt_context_set_limits(tt_context *ctx, int32_t jacobi_sweeps, int64_t 
 tt_status tt_sync(tt_context *ctx);
 
 /* Workspace the context needs for tt_step / tt_round on tensors of capacity `x` with
- * problem `plan` (NULL for tt_round only). */
+ * problem `plan` (NULL for tt_round only).  tt_dot sizes its own: 16 bytes for each entry of up to
+ * 262,144 rows of the first cores, where it forms their products exactly. */
 tt_status tt_workspace_query(tt_context *ctx, const tt_plan *plan, const tt_tensor *x,
                              tt_precision prec, size_t *bytes);
 

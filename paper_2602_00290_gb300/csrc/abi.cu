@@ -58,32 +58,62 @@ bool capturing(cudaStream_t s) {
   return cs != cudaStreamCaptureStatusNone;
 }
 
-tt_status ensure_ws(tt_context* ctx, size_t need) {
+// Provide a workspace of `need` bytes.  The present one is freed only when the larger one is there, or where its own
+// bytes are what the larger one lacks; one that a caller's captured graph uses is never freed.  last: there is no
+// smaller form to fall back to.
+tt_status ensure_ws(tt_context* ctx, size_t need, bool last) {
   if (need <= ctx->ws_bytes) return TT_OK;
   if (capturing(ctx->stream)) return TT_ERR_WORKSPACE;
+  if (!last && ctx->ws_refused > 0 && need >= ctx->ws_refused) return TT_ERR_CUDA;
   if (cudaStreamSynchronize(ctx->stream) != cudaSuccess) return TT_ERR_CUDA;
-  if (ctx->ws) cudaFree(ctx->ws);
-  ctx->ws = nullptr;
-  ctx->ws_bytes = 0;
-  if (cudaMalloc(&ctx->ws, need) != cudaSuccess) return TT_ERR_CUDA;
+  if (ctx->ws_captured) {
+    try {
+      ctx->ws_kept.reserve(ctx->ws_kept.size() + 1);
+    } catch (...) {
+      return TT_ERR_CUDA;
+    }
+  }
+  void* p = nullptr;
+  if (cudaMalloc(&p, need) != cudaSuccess) {
+    (void)cudaGetLastError();
+    size_t left = 0, total = 0;
+    if (!ctx->ws || ctx->ws_captured) return TT_ERR_CUDA;
+    if (!last && (cudaMemGetInfo(&left, &total) != cudaSuccess || left + ctx->ws_bytes < need)) return TT_ERR_CUDA;
+    cudaFree(ctx->ws);
+    ctx->ws = nullptr;
+    ctx->ws_bytes = 0;
+    if (cudaMalloc(&p, need) != cudaSuccess) {
+      (void)cudaGetLastError();
+      return TT_ERR_CUDA;
+    }
+  }
+  if (ctx->ws && ctx->ws_captured) ctx->ws_kept.push_back(ctx->ws);
+  else if (ctx->ws) cudaFree(ctx->ws);
+  ctx->ws = p;
   ctx->ws_bytes = need;
+  ctx->ws_captured = false;
   return TT_OK;
 }
 
 // Size the workspace by a dry run of `fn(Bump&)` and provide it.  Where it cannot be had (a capture in
 // progress on a smaller workspace, or no memory), the call takes the Householder factors instead of
-// the exact Gram products, whose digit records need more (ctx->no_xg, cleared by the next call).
+// the exact Gram products, whose digit records need more (ctx->no_xg, cleared by the next call).  A size that
+// the device refused is not asked for again: each try would wait for the stream.
 template <class F>
 tt_status size_ws(tt_context* ctx, F&& fn) {
   tt_status st = TT_OK;
+  size_t refused = 0;
   for (int attempt = 0; attempt < 2; ++attempt) {
     ctx->no_xg = attempt;
     ttk::Bump dry{nullptr, 0, 0, true};
     st = fn(dry);
     if (st != TT_OK) return st;
-    st = ensure_ws(ctx, dry.need());
-    if (st == TT_OK) return st;
-    (void)cudaGetLastError();
+    st = ensure_ws(ctx, dry.need(), attempt == 1);
+    if (st == TT_OK) {
+      if (refused > dry.need() && (ctx->ws_refused == 0 || refused < ctx->ws_refused)) ctx->ws_refused = refused;
+      return st;
+    }
+    if (st != TT_ERR_WORKSPACE) refused = dry.need();
   }
   return st;
 }
@@ -94,6 +124,7 @@ tt_status with_ws(tt_context* ctx, F&& fn) {
   InstrGuard guard(ctx);
   const tt_status st = size_ws(ctx, fn);
   if (st != TT_OK) return st;
+  if (!ctx->ws_captured && ctx->ws && capturing(ctx->stream)) ctx->ws_captured = true;
   ttk::Bump real{static_cast<char*>(ctx->ws), 0, ctx->ws_bytes, false};
   return fn(real);
 }
@@ -226,7 +257,7 @@ tt_status tt_context_create(tt_context** out, int device, void* stream, size_t w
     return TT_ERR_CUDA;
   }
   cudaMemsetAsync(ctx->ctrl, 0, sizeof(ttk::DevCtrl), ctx->stream);
-  if (workspace_bytes > 0 && ensure_ws(ctx, workspace_bytes) != TT_OK) {
+  if (workspace_bytes > 0 && ensure_ws(ctx, workspace_bytes, true) != TT_OK) {
     cudaFree(ctx->ctrl);
     delete ttk::tune_of(ctx);
     delete static_cast<ttk::Instr*>(ctx->instr);
@@ -249,6 +280,7 @@ tt_status tt_context_destroy(tt_context* ctx) {
   set_device(ctx);
   cudaStreamSynchronize(ctx->stream);
   if (ctx->ws) cudaFree(ctx->ws);
+  for (void* p : ctx->ws_kept) cudaFree(p);
   cudaFree(ctx->ctrl);
   ttk::Instr* in = static_cast<ttk::Instr*>(ctx->instr);
   for (cudaEvent_t e : in->pool) cudaEventDestroy(e);

@@ -188,6 +188,7 @@ tt_status tt_batch_create(tt_context* ctx, int32_t nprob, const tt_plan* const* 
       c.ctrl = b->ctrls + i;
       c.ws = nullptr;
       c.ws_bytes = 0;
+      c.ws_kept.clear();
       c.instr = &b->counts;
       c.tune = &b->tune;
       c.no_xg = attempt;  // where the exact Gram products' digit records do not fit: Householder factors

@@ -4,6 +4,8 @@
 #include <math.h>
 #include <stdint.h>
 
+#include <vector>
+
 #include "tt.h"
 
 namespace ttk {
@@ -131,6 +133,11 @@ struct tt_context {
   int graphs;        // tt_step replays a captured CUDA graph of the step (tt_context_set_graphs)
   void* step_graph;  // the captured step and what it depends on (owned; not shared by batch views)
   long graph_replays, graph_captures, graph_failures;  // since the last diagnostics reset
+  // a caller's graph holds the workspace (it was used under a capture of the stream): it is never freed before the
+  // context; where a larger one took its place it is kept here
+  bool ws_captured = false;
+  std::vector<void*> ws_kept;
+  size_t ws_refused = 0;  // least workspace of the exact products that could not be had (0: none)
   int no_xg = 0;     // the call in progress takes the Householder factors (their workspace is smaller)
   int tensor_cores;  // the call in progress runs TT_PREC_MIXED_3XTF32 (tensor-core contractions)
 };
