@@ -551,6 +551,11 @@ __device__ __forceinline__ void xg_fold(uint32_t ta, int w, uint64_t* release, l
   }
 }
 
+// The ring of stages after `issued` tiles: tiles first .. issued - 1 are the last ones of their stages, and tile u's
+// copies complete the phase of parity (u / nst) & 1 of its stage's mbarrier.
+__host__ __device__ __forceinline__ int xg_last_first(int issued, int nst) { return issued > nst ? issued - nst : 0; }
+__host__ __device__ __forceinline__ unsigned xg_fill_parity(int u, int nst) { return (unsigned)(u / nst) & 1u; }
+
 // Whether MMA group g ends a chunk with tile t (of ntile): the two groups' chunks are half a chunk apart.
 __device__ __forceinline__ bool xg_ends(int g, int t, int ntile) {
   return (t + 1 + g * (kXgChunkTiles / 2)) % kXgChunkTiles == 0 || t == ntile - 1;
@@ -569,7 +574,7 @@ __global__ void __launch_bounds__(kXgThreads, 1)
              int* __restrict__ status) {
   constexpr int W = XgCfg<NS>::W, H = XgCfg<NS>::H;
   extern __shared__ __align__(1024) unsigned char xg_smem[];
-  __shared__ uint64_t full[kXgMaxStage], empty[kXgMaxStage], acc_full[kXgGroups], acc_empty[kXgGroups];
+  __shared__ uint64_t full[kXgMaxStage], empty[kXgMaxStage], acc_full[kXgGroups], acc_empty[kXgGroups], done;
   __shared__ uint32_t tbase, rows_s;
   __shared__ int nsubs, off;
   __shared__ struct {
@@ -598,6 +603,7 @@ __global__ void __launch_bounds__(kXgThreads, 1)
       tc::mbar_init(&acc_full[i], 1);
       tc::mbar_init(&acc_empty[i], 16);
     }
+    tc::mbar_init(&done, 1);
     // a piece of a stage: the rows (digits of columns) of the CTA's blocks one after the other, in eights
     // of po octets each (K-major core matrices without swizzle: LBO 128, SBO 128 po)
     const uint32_t po16 = (uint32_t)ar.po * 16u;
@@ -727,9 +733,9 @@ __global__ void __launch_bounds__(kXgThreads, 1)
                        : (csub[u].arr ? ar.dig[1] : ar.dig[0]) + (size_t)csub[u].c0 * ar.npiece * (ar.po * NS * 16) +
                              (piece[k] + shift) * bytes[k];
     }
-    int st = -1;
+    int st = -1, t = 0;
     uint32_t ph = 1;
-    for (int t = 0; t < ntile; ++t) {
+    for (; t < ntile; ++t) {
       if (++st == nst) {
         st = 0;
         ph ^= 1u;
@@ -761,10 +767,8 @@ __global__ void __launch_bounds__(kXgThreads, 1)
         }
       }
     }
-    // the copies in flight land before the CTA ends (their stages were all consumed otherwise)
-    if (__any_sync(0xffffffffu, lost))
-      for (int st = 0; st < nst; ++st)
-        if (st < ntile) (void)tc::mbar_wait(&full[st], 0, 1L << 16);
+    // the copies in flight land before the CTA ends, whoever gave up (bounded)
+    for (int u = xg_last_first(t, nst); u < t; ++u) (void)tc::mbar_wait(&full[u % nst], xg_fill_parity(u, nst), 1L << 16);
   } else if (lane == 0) {
     // ---- MMAs
     // K steps of two octets; pieces of 1, 2, 3 or 4 steps (3 and 4: one piece a stage)
@@ -844,11 +848,9 @@ __global__ void __launch_bounds__(kXgThreads, 1)
       if (lost) break;
       tc::mma_commit(&empty[st]);
     }
-    if (lost) {
-      // MMAs may still run: wait for them (bounded) before the accumulators are released
-      tc::mma_commit(&empty[0]);
-      (void)tc::mbar_wait(&empty[0], 0, 1L << 16);
-    }
+    // the MMAs end before the accumulators are released, whoever gave up (bounded)
+    tc::mma_commit(&done);
+    if (!tc::mbar_wait(&done, 0, 1L << 16)) lost = true;
   }
   tc::fence_before_sync();
   if (__syncthreads_or(lost) && tid == 0) latch(status, TT_ERR_TIMEOUT);
