@@ -383,8 +383,9 @@ tt_status tt_batch_create(tt_context *ctx, int32_t nprob, const tt_plan *const *
 /* Advance every problem of the batch by nsteps time steps, asynchronously on the context stream.
  * The first batched step runs eagerly (every kernel loaded and configured outside any capture),
  * the next one is captured as a CUDA graph (so neither may be made under an outer stream
- * capture), and every later step is a replay of that graph.  Device-detected errors are
- * latched per problem and reported by tt_batch_sync. */
+ * capture), and every later step is a replay of that graph.  The context's TSQR choice
+ * (tt_context_set_tsqr) counts as it is at the step that runs eagerly or is captured.  Device-detected
+ * errors are latched per problem and reported by tt_batch_sync. */
 tt_status tt_batch_step(tt_batch *b, int32_t nsteps);
 /* Synchronise the context stream; status_out[nprob] (nullable) receives each problem's latched
  * status; returns the first non-OK one. */

@@ -29,11 +29,12 @@ struct tt_batch {
   std::vector<tt_context> sub;  // per-problem views of the context
   ttk::DevCtrl* ctrls;
   void* ws;
+  size_t ws_bytes;
   cudaGraph_t graph;
   cudaGraphExec_t exec;
   bool warmed;  // the first batched step ran eagerly (the graph is captured at the next one)
   cudaEvent_t pre, post;  // order the eager step after / before the context stream's work
-  ttk::TsqrTune tune;  // the context's kernel choice when the batch was made
+  ttk::TsqrTune tune;  // the context's kernel choice that the workspace is sized for (provide_ws)
   ttk::Instr counts;  // launch counts of the captured step (timing off)
 };
 
@@ -62,6 +63,60 @@ void release(tt_batch* b) {
   if (b->ctrls) cudaFree(b->ctrls);
   for (cudaEvent_t e : b->counts.pool) cudaEventDestroy(e);
   delete b;
+}
+
+// Takes over the context's kernel choice and provides every problem's workspace region for it by dry runs.
+tt_status provide_ws(tt_batch* b) {
+  tt_context* ctx = b->ctx;
+  b->tune = *ttk::tune_of(ctx);
+  double rows_all = 0.0;
+  for (int i = 0; i < b->nprob; ++i) rows_all += (double)b->states[i].n[0];
+  ttk::Instr* prev = ttk::g_instr;
+  ttk::g_instr = &b->counts;
+  tt_status st = TT_ERR_CUDA;
+  for (int attempt = 0; attempt < 2 && st == TT_ERR_CUDA; ++attempt) {
+    size_t total = 0;
+    st = TT_OK;
+    for (int i = 0; i < b->nprob && st == TT_OK; ++i) {
+      tt_context& c = b->sub[i];
+      c.no_xg = attempt;  // where the exact Gram products' digit records do not fit: Householder factors
+      // TSQR leaves in proportion to the problem's share of the batch's rows (all problems run at
+      // once): at least 8, at most the single-problem wave
+      const double share = (double)b->states[i].n[0] / rows_all;
+      int cap = (int)(share * 3.0 * ctx->num_sms + 0.5);
+      c.tsqr_leaf_cap = cap < 8 ? 8 : cap;
+      ttk::Bump dry{nullptr, 0, 0, true};
+      st = step_dispatch(&c, b->plans[i], &b->states[i], b->tol[i], b->rmax[i], b->prec, dry);
+      b->ws_off[i] = total;
+      b->ws_len[i] = dry.need();
+      total += (dry.need() + 255) & ~(size_t)255;
+    }
+    if (st != TT_OK) break;
+    if (!b->ws || total > b->ws_bytes) {
+      // (a step may be in flight on the present workspace)
+      if (b->ws) {
+        if (cudaStreamSynchronize(b->origin) != cudaSuccess) {
+          st = TT_ERR_CUDA;
+          break;
+        }
+        cudaFree(b->ws);
+        b->ws = nullptr;
+      }
+      b->ws_bytes = total > 0 ? total : 256;
+      if (cudaMalloc(&b->ws, b->ws_bytes) != cudaSuccess) {
+        b->ws = nullptr;
+        (void)cudaGetLastError();
+        st = TT_ERR_CUDA;
+      }
+    }
+  }
+  ttk::g_instr = prev;
+  if (st != TT_OK) return st;
+  for (int i = 0; i < b->nprob; ++i) {
+    b->sub[i].ws = static_cast<char*>(b->ws) + b->ws_off[i];
+    b->sub[i].ws_bytes = b->ws_len[i];
+  }
+  return TT_OK;
 }
 
 // Issue one batched step on the origin stream (fork into the pool, join back).
@@ -118,6 +173,7 @@ tt_status tt_batch_create(tt_context* ctx, int32_t nprob, const tt_plan* const* 
   b->origin = nullptr;
   b->ctrls = nullptr;
   b->ws = nullptr;
+  b->ws_bytes = 0;
   b->graph = nullptr;
   b->exec = nullptr;
   b->warmed = false;
@@ -173,52 +229,20 @@ tt_status tt_batch_create(tt_context* ctx, int32_t nprob, const tt_plan* const* 
   b->sub.assign(nprob, *ctx);
   b->ws_off.assign(nprob, 0);
   b->ws_len.assign(nprob, 0);
-  size_t total = 0;
-  double rows_all = 0.0;
-  for (int i = 0; i < nprob; ++i) rows_all += (double)b->states[i].n[0];
-  // the kernel choice as it is now: the workspace below is sized for it
-  b->tune = *ttk::tune_of(ctx);
-  ttk::Instr* prev = ttk::g_instr;
-  ttk::g_instr = &b->counts;
-  for (int attempt = 0; attempt < 2 && !b->ws; ++attempt) {
-    total = 0;
-    for (int i = 0; i < nprob; ++i) {
-      tt_context& c = b->sub[i];
-      c.stream = b->streams[b->stream_of[i]];
-      c.ctrl = b->ctrls + i;
-      c.ws = nullptr;
-      c.ws_bytes = 0;
-      c.ws_kept.clear();
-      c.instr = &b->counts;
-      c.tune = &b->tune;
-      c.no_xg = attempt;  // where the exact Gram products' digit records do not fit: Householder factors
-      c.coop_grid_max = 1;
-      // TSQR leaves in proportion to the problem's share of the batch's rows (all problems run at
-      // once): at least 8, at most the single-problem wave
-      const double share = (double)b->states[i].n[0] / rows_all;
-      int cap = (int)(share * 3.0 * ctx->num_sms + 0.5);
-      c.tsqr_leaf_cap = cap < 8 ? 8 : cap;
-      ttk::Bump dry{nullptr, 0, 0, true};
-      tt_status st = step_dispatch(&c, b->plans[i], &b->states[i], b->tol[i], b->rmax[i], prec, dry);
-      if (st != TT_OK) {
-        ttk::g_instr = prev;
-        release(b);
-        return st;
-      }
-      b->ws_off[i] = total;
-      b->ws_len[i] = dry.need();
-      total += (dry.need() + 255) & ~(size_t)255;
-    }
-    if (cudaMalloc(&b->ws, total > 0 ? total : 256) != cudaSuccess) {
-      b->ws = nullptr;
-      (void)cudaGetLastError();
-    }
-  }
-  ttk::g_instr = prev;
-  if (!b->ws) { release(b); return TT_ERR_CUDA; }
   for (int i = 0; i < nprob; ++i) {
-    b->sub[i].ws = static_cast<char*>(b->ws) + b->ws_off[i];
-    b->sub[i].ws_bytes = b->ws_len[i];
+    tt_context& c = b->sub[i];
+    c.stream = b->streams[b->stream_of[i]];
+    c.ctrl = b->ctrls + i;
+    c.ws = nullptr;
+    c.ws_bytes = 0;
+    c.ws_kept.clear();
+    c.instr = &b->counts;
+    c.tune = &b->tune;
+    c.coop_grid_max = 1;
+  }
+  if (const tt_status st = provide_ws(b); st != TT_OK) {
+    release(b);
+    return st;
   }
   if (cudaStreamSynchronize(ctx->stream) != cudaSuccess) { release(b); return TT_ERR_CUDA; }
   *out = b;
@@ -229,6 +253,9 @@ tt_status tt_batch_step(tt_batch* b, int32_t nsteps) {
   if (!b || nsteps < 0) return TT_ERR_ARG;
   tt_context* ctx = b->ctx;
   if (cudaSetDevice(ctx->device) != cudaSuccess) return TT_ERR_CUDA;
+  if (!b->exec && nsteps > 0 && (!b->ws || ttk::tune_of(ctx)->epoch != b->tune.epoch)) {
+    if (const tt_status st = provide_ws(b); st != TT_OK) return st;
+  }
   if (!b->exec && !b->warmed && nsteps > 0) {
     // The first batched step runs eagerly: every kernel is loaded and has its shared-memory
     // limit set outside any capture; the graph is captured at the next step.
