@@ -13,9 +13,6 @@
 // the rotation's angle is formed in FP32 (the rotation itself is orthogonal to FP64 round-off; an angle
 // accurate to 2^-22 only costs a sweep's final factor).
 #pragma once
-#include <map>
-#include <mutex>
-
 #include "common.cuh"
 #include "instr.cuh"
 #include "xchol.cuh"
@@ -25,11 +22,11 @@ namespace ttk {
 constexpr int kJcMaxN = 256;
 constexpr int kJcMaxB = 16;  // columns of a block (a warp per pair)
 
-// Cluster size: blocks of at most 16 columns, small enough that an inner round is one or two pairs per
-// sub-partition.  FP64 takes more SMs for its slow pipe.
+// Cluster size, up to the eight CTAs that every cluster launch may have: blocks of at most 16 columns, small enough
+// that an inner round is one or two pairs per sub-partition.  FP64 takes more SMs for its slow pipe up to 64 columns.
 template <typename T>
 inline int jc_cluster(int n) {
-  if (sizeof(T) == 8) return n <= 8 ? 1 : n <= 16 ? 2 : n <= 40 ? 4 : n <= 80 ? 8 : 16;
+  if (sizeof(T) == 8) return n <= 8 ? 1 : n <= 16 ? 2 : n <= 40 ? 4 : 8;
   return n <= 32 ? 1 : n <= 64 ? 4 : 8;
 }
 __host__ __device__ inline int jc_ld(int n) { return (n + 31) & ~31; }
@@ -417,9 +414,10 @@ __global__ void __launch_bounds__(512) k_jacobi_cl(int n, const double* __restri
 }
 
 template <typename T, int E>
-inline tt_status launch_jacobi_cl_e(cudaStream_t s, int n, int C, const double* R, double* U, double* raw, int* perm,
-                                    float drop, DevCtrl* ctrl) {
+inline tt_status launch_jacobi_cl_e(cudaStream_t s, int n, const double* R, double* U, double* raw, int* perm, float drop,
+                                    DevCtrl* ctrl) {
   auto kern = k_jacobi_cl<T, E>;
+  const int C = jc_cluster<T>(n);
   size_t smem = jc_smem_bytes<T>(n, C);
   if (smem < sizeof(double) * (size_t)n) smem = sizeof(double) * (size_t)n;
   if (const tt_status a = smem_optin(kern, smem); a != TT_OK) return a;
@@ -442,60 +440,16 @@ inline tt_status launch_jacobi_cl_e(cudaStream_t s, int n, int C, const double* 
   count_launch();
   return TT_OK;
 }
-// Whether clusters of 16 CTAs of the kernel can run (asked once per kernel and context).
-template <typename T, int E>
-inline bool jc_wide_ok(int n) {
-  // per CUDA context: one that is destroyed and re-created needs the attribute again
-  static std::mutex mu;
-  static std::map<unsigned long long, bool> done;
-  const unsigned long long cid = current_context_id();
-  std::lock_guard<std::mutex> lock(mu);
-  const auto it = done.find(cid);
-  if (cid != 0 && it != done.end()) return it->second;
-  const bool ok = [&] {
-    auto kern = k_jacobi_cl<T, E>;
-    if (cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess) {
-      (void)cudaGetLastError();
-      return false;
-    }
-    cudaLaunchConfig_t cfg{};
-    cfg.gridDim = dim3(16);
-    cfg.blockDim = dim3(256);
-    cfg.dynamicSmemBytes = 48 * 1024;
-    cudaLaunchAttribute at{};
-    at.id = cudaLaunchAttributeClusterDimension;
-    at.val.clusterDim.x = 16;
-    at.val.clusterDim.y = at.val.clusterDim.z = 1;
-    cfg.attrs = &at;
-    cfg.numAttrs = 1;
-    int nc = 0;
-    if (cudaOccupancyMaxActiveClusters(&nc, kern, &cfg) != cudaSuccess) {
-      (void)cudaGetLastError();
-      return false;
-    }
-    return nc > 0;
-  }();
-  (void)n;
-  if (cid != 0) done[cid] = ok;
-  return ok;
-}
-template <typename T, int E>
-inline tt_status launch_jacobi_cl_n(cudaStream_t s, int n, const double* R, double* U, double* raw, int* perm, float drop,
-                                    DevCtrl* ctrl) {
-  int C = jc_cluster<T>(n);
-  if (C == 16 && !jc_wide_ok<T, E>(n)) C = 8;
-  return launch_jacobi_cl_e<T, E>(s, n, C, R, U, raw, perm, drop, ctrl);
-}
 // U, raw and perm of the n x n factor R (see k_jacobi_cl) on stream s.
 template <typename T>
 tt_status launch_jacobi_cl(cudaStream_t s, int n, const double* R, double* U, double* raw, int* perm, DevCtrl* ctrl) {
   // rows below drop ||R||_F together change R by less than sqrt(n) drop ||R||_F: below the rounding of R
   const float drop = sizeof(T) == 4 ? 9.31322574615478515625e-10f : 8.6736173798840355e-19f;  // 2^-30, 2^-60
   if (n > kJcMaxN) return TT_ERR_UNSUPPORTED;
-  if (n <= 32) return launch_jacobi_cl_n<T, 1>(s, n, R, U, raw, perm, drop, ctrl);
-  if (n <= 64) return launch_jacobi_cl_n<T, 2>(s, n, R, U, raw, perm, drop, ctrl);
-  if (n <= 160) return launch_jacobi_cl_n<T, 5>(s, n, R, U, raw, perm, drop, ctrl);
-  return launch_jacobi_cl_n<T, 8>(s, n, R, U, raw, perm, drop, ctrl);
+  if (n <= 32) return launch_jacobi_cl_e<T, 1>(s, n, R, U, raw, perm, drop, ctrl);
+  if (n <= 64) return launch_jacobi_cl_e<T, 2>(s, n, R, U, raw, perm, drop, ctrl);
+  if (n <= 160) return launch_jacobi_cl_e<T, 5>(s, n, R, U, raw, perm, drop, ctrl);
+  return launch_jacobi_cl_e<T, 8>(s, n, R, U, raw, perm, drop, ctrl);
 }
 
 }  // namespace ttk
