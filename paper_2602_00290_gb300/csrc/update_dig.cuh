@@ -42,13 +42,18 @@ constexpr long kUdMinRows = 1024;
 constexpr long kUdMinRowsTc = 4096;
 constexpr int kUdDead = 1 << 20;                 // column scale that makes every digit zero
 constexpr int kUdMinExp = -8000;                 // row scale of a zero row
+// Rows of FP32 storage in an FP32 pass whose scales (row + column) reach below kUdPowMin, where the power of two of an
+// entry leaves FP32 (rows below about 1e-29): their entries are multiplied by 2^kUdRaise first, and the row's scale
+// is stored as much larger.  Not where the columns' sizes differ by 2^kUdWide or more: the raised entries could
+// leave FP32 at the other end, and rows end at kUdPowMin.
+constexpr int kUdRaised = 1 << 22, kUdRaise = 28, kUdPowMin = -98, kUdWide = 180;
 
 // Scales of a pass and where its weights' digits go (workspace).
 struct UdBufs {
   int* cexp = nullptr;        // [ncap] size of each column (launch_ud_scales, launch_ud_scales_cols)
   unsigned long long* slots = nullptr;  // [columns] largest entries (launch_ud_scales_cols)
   short* rho = nullptr;       // [nrows] exponent of a storage row (stencil passes)
-  int* rinfo = nullptr;       // [nrows] scale of a row of the pass (16 bits), neighbour flags from bit 16
+  int* rinfo = nullptr;       // [nrows] scale of a row of the pass (16 bits), neighbour flags from bit 16, kUdRaised
   unsigned char* w = nullptr; // digits of the weights, exponents
 };
 
@@ -156,22 +161,47 @@ static __global__ void __launch_bounds__(256) k_ud_slotexp(int ncol, int extra0,
 }
 
 __device__ __forceinline__ int ud_exp(double x) { return (int)((__double_as_longlong(x) >> 52) & 0x7ff) - 1023; }
-__device__ __forceinline__ int ud_exp(float x) { return (int)((__float_as_uint(x) >> 23) & 0xff) - 127; }
+__device__ __forceinline__ int ud_exp(float x) { return max((int)((__float_as_uint(x) >> 23) & 0xff), 1) - 127; }
+// Row information of scale m and neighbour flags f; raise: an FP32 pass over FP32 storage, amin, amax: the smallest and
+// largest column.
+__device__ __forceinline__ int ud_rinfo(int m, unsigned f, bool raise, int amin, int amax) {
+  const bool up = raise && amax - amin < kUdWide && m + amin < kUdPowMin && m > kUdMinExp + 1;
+  return (int)((f << 16) | (up ? (unsigned)kUdRaised : 0u) | ((unsigned)(up ? m + kUdRaise : m) & 0xffffu));
+}
+__device__ __forceinline__ int ud_row_scale(int inf) {
+  return (int)(short)(inf & 0xffff) - ((inf & kUdRaised) ? kUdRaise : 0);
+}
+__device__ __forceinline__ float ud_row_raise(int inf) {
+  return __int_as_float(0x3f800000 + ((inf & kUdRaised) ? kUdRaise << 23 : 0));
+}
+
+// Smallest and largest of the live columns (kUdDead, 0 where there are none); a full warp.
+__device__ __forceinline__ void ud_col_range(const int* cexp, int ncol, const LivePattern& lp, int r, int& amin,
+                                             int& amax) {
+  amin = kUdDead;
+  amax = -kUdDead;
+  for (int c = threadIdx.x & 31; c < ncol; c += 32)
+    if (lp.live(c, r)) {
+      amin = min(amin, cexp[c]);
+      amax = max(amax, cexp[c]);
+    }
+  amin = __reduce_min_sync(0xffffffffu, amin);
+  amax = __reduce_max_sync(0xffffffffu, amax);
+}
 
 // rho of the rows of a storage matrix: largest exponent of an entry against its column's; eight lanes take
 // a row (rows of 33 columns waste little), a warp 16 rows at a time.
 template <typename S, typename O>
 __global__ void __launch_bounds__(256) k_ud_rows(const S* __restrict__ A, long ld, LivePattern lp, int ncol, long nrows,
-                                                 const int* __restrict__ cexp, O* __restrict__ out) {
+                                                 const int* __restrict__ cexp, O* __restrict__ out, bool raise) {
   const int lane = threadIdx.x & 31, l8 = lane & 7, g = lane >> 3;
   const long warp = ((long)blockIdx.x * blockDim.x + threadIdx.x) >> 5, nw = ((long)gridDim.x * blockDim.x) >> 5;
   const int r = lp.r_ptr ? *lp.r_ptr : lp.rcap;
-  int amin = kUdDead;
-  for (int c = l8; c < ncol; c += 8)
-    if (lp.live(c, r)) amin = min(amin, cexp[c]);
-  amin = __reduce_min_sync(0xffffffffu, amin);
-  // rows below the normal numbers of the storage against their columns share one scale
-  const int low = amin == kUdDead ? kUdMinExp : (sizeof(S) == 4 ? -98 : -950) - amin;
+  int amin, amax;
+  ud_col_range(cexp, ncol, lp, r, amin, amax);
+  // rows at the end of the storage's numbers against their columns share one scale
+  const int low = amin == kUdDead ? kUdMinExp
+                                  : (sizeof(S) == 8 ? -950 : amax - amin < kUdWide ? -126 : kUdPowMin) - amin;
   for (long k0 = 16 * warp; k0 < nrows; k0 += 16 * nw) {
     int m[4];
 #pragma unroll
@@ -193,7 +223,7 @@ __global__ void __launch_bounds__(256) k_ud_rows(const S* __restrict__ A, long l
     }
     const int v = l8 == 0 ? m[0] : l8 == 1 ? m[1] : l8 == 2 ? m[2] : m[3];
     const long k = k0 + 4 * l8 + g;
-    if (l8 < 4 && k < nrows) out[k] = sizeof(O) == 2 ? (O)v : (O)(v & 0xffff);
+    if (l8 < 4 && k < nrows) out[k] = sizeof(O) == 2 ? (O)v : (O)ud_rinfo(v, 0u, raise, amin, amax);
   }
 }
 
@@ -202,8 +232,10 @@ __global__ void __launch_bounds__(256) k_ud_rows(const S* __restrict__ A, long l
 template <typename S>
 __global__ void __launch_bounds__(256) k_ud_info(const __grid_constant__ SrcStencil<S> src, LivePattern lp, long nrows,
                                                  const int* __restrict__ cexp, const short* __restrict__ rho,
-                                                 int* __restrict__ rinfo) {
+                                                 int* __restrict__ rinfo, bool raise) {
   const long k = (long)blockIdx.x * blockDim.x + threadIdx.x;
+  int amin, amax;
+  ud_col_range(cexp, src.rcap, LivePattern{lp.r_ptr, lp.rcap, 1, 0}, lp.r_ptr ? *lp.r_ptr : lp.rcap, amin, amax);
   if (k >= nrows) return;
   int m = rho[k];
   unsigned f = 0u;
@@ -225,7 +257,7 @@ __global__ void __launch_bounds__(256) k_ud_info(const __grid_constant__ SrcSten
     const double v = at_face ? src.bcval[e * src.G + (int)((unsigned)k % (unsigned)src.G)] : 0.0;
     if (v != 0.0) m = max(m, ud_exp(v) - cexp[(src.nterm + 1) * src.rcap + e]);
   }
-  rinfo[k] = (int)((f << 16) | ((unsigned)m & 0xffffu));
+  rinfo[k] = ud_rinfo(m, f, raise, amin, amax);
 }
 
 // Digits of the weights, one block per output column n, in the layout of the B operand (K-major core
@@ -300,9 +332,9 @@ __device__ __forceinline__ long long ud_fix(float x, int scale, int& top) {
   const unsigned b = __float_as_uint(x);
   const int e = (int)((b >> 23) & 0xff);
   top = max(top, e);
-  const unsigned long long m = e ? ((unsigned long long)((b & 0x7fffffu) | 0x800000u) << 39) : 0ull;
+  const unsigned long long m = (unsigned long long)((b & 0x7fffffu) | (e ? 0x800000u : 0u)) << 39;
   const long long sg = (long long)((int)b >> 31);
-  return ((long long)(m >> min(max(scale + 128 - e, 1), 63)) ^ sg) - sg;
+  return ((long long)(m >> min(max(scale + 128 - max(e, 1), 1), 63)) ^ sg) - sg;
 }
 // FP32 entries of an FP32 pass: a power of two (zero for dead columns) and a conversion, rounded to nearest.
 __device__ __forceinline__ float ud_pow(int scale) { return __int_as_float(max(156 - scale, 0) << 23); }
@@ -364,9 +396,9 @@ __device__ __forceinline__ void ud_fix2(const UdPair<S>& x, int2 a, int r, V& v0
   if (top == (sizeof(S) == 4 ? 255 : 2047))
     bad = bad || (!isfinite(x.a) && a.x != kUdDead) || (!isfinite(x.b) && a.y != kUdDead);
 }
-__device__ __forceinline__ void ud_fix2f(float x0, float x1, float f0, float f1, int& v0, int& v1, bool& bad) {
-  v0 = __float2int_rn(x0 * f0);
-  v1 = __float2int_rn(x1 * f1);
+__device__ __forceinline__ void ud_fix2f(float x0, float x1, float up, float f0, float f1, int& v0, int& v1, bool& bad) {
+  v0 = __float2int_rn((x0 * up) * f0);
+  v1 = __float2int_rn((x1 * up) * f1);
   const float t = fmaf(x1, 0.0f, x0 * 0.0f);
   if (t != 0.0f) bad = bad || (!isfinite(x0) && f0 != 0.0f) || (!isfinite(x1) && f1 != 0.0f);
 }
@@ -442,10 +474,11 @@ __device__ __forceinline__ void ud_digits(const SrcStencil<S>& s, const LivePatt
           y = UdPair<S>{y.a - c.a, y.b - c.b};
         }
         const int2 ay = u < np ? a1 : a0;
+        const float up = ud_row_raise(inf[g]);
         int v0, v1;
-        ud_fix2f(x.a, x.b, ud_pow(r + a0.x), ud_pow(r + a0.y), v0, v1, bad);
+        ud_fix2f(x.a, x.b, up, ud_pow(r + a0.x), ud_pow(r + a0.y), v0, v1, bad);
         ud_store2<NS>(v0, v1, at + 128 * g);
-        ud_fix2f(y.a, y.b, ud_pow(r + ay.x), ud_pow(r + ay.y), v0, v1, bad);
+        ud_fix2f(y.a, y.b, up, ud_pow(r + ay.x), ud_pow(r + ay.y), v0, v1, bad);
         ud_store2<NS>(v0, v1, at + 2048 + 128 * g);
       }
       return;
@@ -474,7 +507,7 @@ __device__ __forceinline__ void ud_digits(const SrcStencil<S>& s, const LivePatt
     }
   } else {
     for (int g = 0; g < 4; ++g) {
-      const int r = (int)(short)(inf[g] & 0xffff);
+      const int r = ud_row_scale(inf[g]);
       const unsigned f = (unsigned)inf[g] >> 16;
       UdPair<double> x{0.0, 0.0};
       for (int e = c2; e < c2 + 2 && e < lp.nextra; ++e) {
@@ -499,9 +532,10 @@ __device__ __forceinline__ void ud_digits(const SrcRows<S>&, const LivePattern&,
     const int r = (int)(short)(inf[g] & 0xffff);
     typename std::conditional<NS == 4, int, long long>::type v0, v1;
     if constexpr (NS == 4 && sizeof(S) == 4) {
-      ud_fix2f(w.x[g].a, w.x[g].b, ud_pow(r + a0.x), ud_pow(r + a0.y), v0, v1, bad);
+      const float up = ud_row_raise(inf[g]);
+      ud_fix2f(w.x[g].a, w.x[g].b, up, ud_pow(r + a0.x), ud_pow(r + a0.y), v0, v1, bad);
       ud_store2<NS>(v0, v1, at + 128 * g);
-      ud_fix2f(w.y[g].a, w.y[g].b, ud_pow(r + a1.x), ud_pow(r + a1.y), v0, v1, bad);
+      ud_fix2f(w.y[g].a, w.y[g].b, up, ud_pow(r + a1.x), ud_pow(r + a1.y), v0, v1, bad);
     } else {
       ud_fix2<NS>(w.x[g], a0, r, v0, v1, bad);
       ud_store2<NS>(v0, v1, at + 128 * g);
@@ -648,7 +682,7 @@ __global__ void __launch_bounds__(ud_threads(NS), 1)
     for (long tile = blockIdx.x; tile < ntiles; tile += gridDim.x, ++it) {
       const int buf = (int)(it & 1);
       const long k0 = tile * 128 + 32 * q, k = k0 + lane;
-      const int r = k < nrows ? (int)(short)(rinfo[k] & 0xffff) : kUdMinExp;
+      const int r = k < nrows ? ud_row_scale(rinfo[k]) : kUdMinExp;
       // the two warps of a quarter leave together
       if (!tc::pair_and(1 + q, tc::mbar_wait(&dfull[buf], (uint32_t)((it >> 1) & 1)))) {
         lost = true;
@@ -947,12 +981,13 @@ tt_status launch_update_dig(cudaStream_t s, int num_sms, const Src& src, LivePat
   const long rb = (nrows + 127) / 128, gr = rb < 16L * num_sms ? rb : 16L * num_sms;
   if constexpr (XgElem<Src>::stencil) {
     LivePattern lz{lp.r_ptr, lp.rcap, 1, 0};
-    k_ud_rows<S, short><<<(unsigned)gr, 256, 0, s>>>(src.Z, src.ldz, lz, src.rcap, nrows, ub.cexp, ub.rho);
+    k_ud_rows<S, short><<<(unsigned)gr, 256, 0, s>>>(src.Z, src.ldz, lz, src.rcap, nrows, ub.cexp, ub.rho, false);
     count_launch();
-    k_ud_info<S><<<(unsigned)((nrows + 255) / 256), 256, 0, s>>>(src, lp, nrows, ub.cexp, ub.rho, ub.rinfo);
+    k_ud_info<S><<<(unsigned)((nrows + 255) / 256), 256, 0, s>>>(src, lp, nrows, ub.cexp, ub.rho, ub.rinfo, NS == 4 && sizeof(S) == 4);
     count_launch();
   } else {
-    k_ud_rows<S, int><<<(unsigned)gr, 256, 0, s>>>(src.A, src.ld, lp, lp.ncap(), nrows, ub.cexp, ub.rinfo);
+    k_ud_rows<S, int><<<(unsigned)gr, 256, 0, s>>>(src.A, src.ld, lp, lp.ncap(), nrows, ub.cexp, ub.rinfo,
+                                                          NS == 4 && sizeof(S) == 4);
     count_launch();
   }
   const long ntiles = (nrows + 127) / 128, grid = num_sms < ntiles ? num_sms : ntiles;

@@ -259,8 +259,9 @@ inline int xg_stages(const XgPlan& pl, int oct = kXgStageOct) {
 __host__ __device__ inline int xg_unit(unsigned long long maxbits, int NS) {
   return ((int)((maxbits >> 52) & 0x7ff) - 1022) - (8 * NS - 2);
 }
-// round(x 2^-U), U folded into the shift constant K (see xg_shift_const).  An exponent field of zero
-// (zero, denormals) gives 0; Inf and NaN give some in-range integer.
+// round(x 2^-U), U folded into the shift constant K (see xg_shift_const).  Zero and FP64's subnormal numbers (an
+// exponent field of zero; their squares vanish in FP64) give 0, FP32's are taken as FP64 numbers; Inf and NaN give
+// some in-range integer.
 __device__ __forceinline__ long long xg_fix(double x, int K) {
   const unsigned long long b = (unsigned long long)__double_as_longlong(x);
   const int e = (int)((b >> 52) & 0x7ff);
@@ -272,7 +273,8 @@ __device__ __forceinline__ long long xg_fix(double x, int K) {
 __device__ __forceinline__ long long xg_fix(float x, int K) {
   const unsigned b = __float_as_uint(x);
   const int e = (int)((b >> 23) & 0xff);
-  const unsigned long long m = e ? ((unsigned long long)((b & 0x7fffffu) | 0x800000u) << 39) : 0ull;
+  if (e == 0) return b << 1 ? xg_fix((double)x, K + 896) : 0;
+  const unsigned long long m = (unsigned long long)((b & 0x7fffffu) | 0x800000u) << 39;
   const int sh = min(max(K - e, 0), 63);
   const long long r = (long long)(((m >> sh) + 1ull) >> 1);
   return (int)b < 0 ? -r : r;
