@@ -289,6 +289,23 @@ def run_reference(args):
     return 0
 
 
+def update_digit_products(precision, rows, rcap, nax=2, nextra=0):
+    """Digit products of an entry that the update pass over the transport sum keeps when it runs from digits on the
+    tensor cores, None where another kernel runs (the library's rule: update_dig_fits and take_ud)."""
+    ns, size = (8, 8) if precision == "fp64" else (4, 4)
+    kp = (rcap + 15) // 16 * 16
+    groups = (rcap + 7) // 8
+    steps = (groups + 1) // 2 + nax * groups + (1 if nextra else 0)
+    fixed = steps * 32 * ns * kp + 4 * (16 * steps + kp) + 256 * size + size * (kp + 128 * (kp + 1)) + 16
+    stages = (225 * 1024 - fixed) // (ns * 4096) if fixed < 225 * 1024 else 0
+    if not 1024 <= rows < 1 << 31 or ns * kp > 256 or steps > 64 or stages < 3:
+        return None
+    if precision == "mixed_3xtf32" and rows < 4096 and rcap in (8, 16, 32):
+        return None  # k_update_tc (FP32 storage)
+    orders = 5 if ns == 4 and 5 * kp <= 256 else ns
+    return sum(1 for i in range(ns) for j in range(ns) if i + j < orders)
+
+
 def time_precision(tt, torch, ctx, plan, wl, args, precision, dist, clocks_index, peaks, rounding="tsqr"):
     """W warm-up then K timed tt_step calls for one precision; returns (line fields, state)."""
     ctx.set_rounding(rounding)
@@ -421,20 +438,27 @@ def time_precision(tt, torch, ctx, plan, wl, args, precision, dist, clocks_index
                            "peak_source": ("FP64" if precision == "fp64" else "FP32") + " FMA pipe, " + pk["source"] +
                                           " in this run (tt_peak_probe)",
                            "share": (kms["tsqr_leaf"] / nb) / (total_ms / args.steps) if total_ms else None}
-    # the first update pass (Z_new = Z_sum W over the transport sum, K = R1, N = r'): from digits on the
-    # tensor cores (products of digits i + j below the orders kept: 13 for FP32 passes, 36 for FP64)
+    # the first update pass (Z_new = Z_sum W over the transport sum, K = R1, N = r')
     up_flops = 0.0
     for i in range(nb):
         up_flops += 2.0 * N * (5 * b_ranks[i][1]) * b_ranks[i + 1][1]
     if kms["update"] > 0:
         up_alg = up_flops / (kms["update"] / 1e3) / 1e12
-        pairs = 36 if precision == "fp64" else 13
-        out["roofline_update"] = {
-            "kernel": "k_update_dig (tcgen05 kind::f16, base-256 digits) with its row and weight scales",
-            "bound": "tensor", "achieved": pairs * up_alg, "peak": f16_peak, "unit": "TFLOP/s",
-            "frac": pairs * up_alg / f16_peak, "algorithmic_tflops": up_alg,
-            "flops_per_launch": "%d x 2 N_Z R1 r' kind::f16 flops (digit products kept)" % pairs,
-            "peak_source": f16_source, "ms_per_launch": kms["update"] / nb}
+        pairs = update_digit_products(precision, N, x.rcap[1])
+        out["roofline_update"] = {"algorithmic_tflops": up_alg, "ms_per_launch": kms["update"] / nb, "unit": "TFLOP/s"}
+        if pairs:
+            out["roofline_update"].update(
+                kernel="k_update_dig (tcgen05 kind::f16, base-256 digits) with its row and weight scales",
+                bound="tensor", achieved=pairs * up_alg, peak=f16_peak, frac=pairs * up_alg / f16_peak,
+                flops_per_launch="%d x 2 N_Z R1 r' kind::f16 flops (digit products kept)" % pairs, peak_source=f16_source)
+        else:
+            out["roofline_update"].update(
+                kernel="k_update_tc (split TF32)" if precision == "mixed_3xtf32" and x.rcap[1] in (8, 16, 32) else
+                       "k_update (FP64 FMA)" if precision == "fp64" else "k_update_blk or k_update (FP32 FMA)",
+                bound="alu", achieved=up_alg, peak=peak, frac=up_alg / peak,
+                flops_per_launch="2 N_Z R1 r' (R1 = 5 r)",
+                peak_source=("FP64" if precision == "fp64" else "FP32") + " FMA pipe, " + pk["source"] +
+                            " in this run (tt_peak_probe)")
     ctx.set_rounding("tsqr")
     return out, x, energy
 
