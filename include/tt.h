@@ -128,7 +128,7 @@ typedef struct tt_context tt_context;
 /* Factor of the merged core in the first sweep of every rounding (tt_round, tt_step).
  * TT_ROUND_TSQR: the triangular factor of the SVD-based rounding of Sec. 3.1 (the default), to the
  * accuracy of the arithmetic: from exact Gram products of the columns on the tensor cores (integer
- * digits, a Cholesky factor in 128-bit fixed point), or by Householder TSQR where
+ * digits, a Cholesky factor in 128-bit fixed point for FP64 passes, 64-bit for FP32 ones), or by Householder TSQR where
  * tt_context_set_tsqr chose its kernels, where the shape does not fit the former, or where its larger
  * workspace cannot be had.
  * TT_ROUND_GRAM: Gram-based (Sec. 3.1 lists it among the solver's rounding methods): the FP64 Gram
@@ -164,13 +164,14 @@ tt_status tt_context_destroy(tt_context *ctx);
  * later call records CUDA events on the context stream around its hot kernels, grouped as
  * TT_TIMER_* categories.  Launch counts are always collected. */
 typedef enum {
-  TT_TIMER_TSQR_LEAF = 0,   /* leaf pass of the tall-skinny QR over the merged core (the
-                               transport sum in tt_step, the tensor itself in tt_round)    */
-  TT_TIMER_TSQR_MERGE = 1,  /* merge tree of the R factors                                 */
+  TT_TIMER_TSQR_LEAF = 0,   /* exact products of the merged core's columns, or the leaf pass of its
+                               tall-skinny QR (the transport sum in tt_step, the tensor itself in
+                               tt_round)                                                   */
+  TT_TIMER_TSQR_MERGE = 1,  /* Cholesky factor of the products, or the merge tree of the R factors */
   TT_TIMER_SMALL = 2,       /* small-core sweep (QRs, Jacobi SVDs, rank decisions)         */
   TT_TIMER_UPDATE = 3,      /* update pass Z_new = Z_sum W (and the fused source step)     */
   TT_TIMER_OTHER = 4,       /* everything else (counted only)                              */
-  TT_TIMER_TSQR_LEAF_SOURCE = 5, /* leaf pass over the source sum (second rounding of tt_step) */
+  TT_TIMER_TSQR_LEAF_SOURCE = 5, /* products or leaf pass over the source sum (second rounding of tt_step) */
   TT_TIMER_UPDATE_SOURCE = 6     /* update pass of the second rounding of tt_step (the source sum);
                                     TT_TIMER_UPDATE then times the first one alone              */
 } tt_timer;
@@ -276,7 +277,7 @@ tt_status tt_context_diagnostics(tt_context *ctx, int64_t *out, int n, int reset
  * paper has no counterpart).  jacobi_sweeps > 0 caps the sweeps of every FP64 one-sided Jacobi
  * SVD (default 40): an SVD still rotating at the cap latches TT_ERR_TIMEOUT.  barrier_spins > 0
  * caps the spins of one wait at the grid-wide barrier of a cooperative kernel (default 2^24 spins
- * of about 64 ns each).  barrier_extra > 0 makes every such barrier wait for that many arrivals
+ * of about 64 ns each) and of one wait of the cluster Jacobi for its other CTAs (2^24 tries).  barrier_extra > 0 makes every such barrier wait for that many arrivals
  * beyond the grid, which never come, so every wait runs out: the kernel latches TT_ERR_TIMEOUT,
  * all its CTAs leave, and the context stays usable (the next cooperative launch starts a fresh
  * barrier).  0 restores a default.  Synchronous (one small host-to-device copy); a step graph

@@ -2,15 +2,15 @@
 // balanced base 256 (xgram.cuh), FP32 passes with 4 digits, FP64 passes with 8.
 //
 // The columns x_c of a row are the centre row, its differences with the neighbours (exact subtractions, as in
-// k_update_blk) and the inflow columns.  With a power of two per column (2^a_c, the size of the
-// column in the triangular factor) and one per row (2^r), v_c = round(x_c 2^-(r + a_c) ..) keeps 2^-30 (FP32)
+// k_update_blk) and the inflow columns.  With a power of two per column (2^a_c, its size: in the
+// triangular factor, or its largest entry) and one per row (2^r), v_c = round(x_c 2^-(r + a_c) ..) keeps 2^-30 (FP32)
 // or 2^-62 (FP64) of the row's largest scaled entry: rows and columns of any grading keep more bits than
 // the arithmetic that the pass stands for.  The weights w_cn 2^a_c get a power of two per output column.  Then
 //   sum_c v_c w_cn = sum_o 256^(2 NS - 2 - o) A_o,   A_o = sum_{i + j = o} sum_c d_j e_i
 // for digits d_j of v and e_i of w, and the A_o are integers below 2^24 in the FP32 accumulators of
 // tcgen05.mma.kind::f16, exact except in the lowest orders of wide FP64 passes (where a lost bit is 2^-60 of the
 // result).  Orders from NS (FP32: NS + 1 where the accumulators fit) on are dropped: 2^-28 (2^-36) and 2^-59
-// of the largest product.  For digit j of the rows the operand B is [e_0 | .. | e_(NS-1-j)], a prefix
+// of the largest product; the read-back rounds once.  For digit j of the rows the operand B is [e_0 | .. | e_(NS-1-j)], a prefix
 // of one resident tile, and its products land in the orders j, j + 1, ..: one MMA does all of them.
 //
 // Eight or twelve warps form the digits (a row and 16 columns each) in a ring of K steps, one thread issues the
@@ -33,12 +33,14 @@ __host__ __device__ constexpr int ud_prod(int ns) { return ns == 4 ? 12 : 8; }
 __host__ __device__ constexpr int ud_threads(int ns) { return 32 * (kUdEpi + ud_prod(ns) + 1); }
 constexpr int kUdMaxSlots = 8;
 constexpr int kUdMaxUnits = 64;                  // K steps of 16 columns
-// Passes of fewer rows stay with the other kernels.  Both updates of a plane step, all launches, digits against
-// before: 4,096 rows, rank 32: FP64 69 / 114 us, FP32 50 / 83 us; rank 8: 43 / 68, 35 / 58 us; 65,536 rows, rank 32:
+// Passes of fewer rows stay with the other kernels (eight tiles leave most SMs idle there).  Both updates of a plane
+// step, all launches, digits against before: 1,024 rows, rank 32: FP64 78 / 123 us, FP32 60 / 82 us; rank 8: 59 / 75,
+// 46 / 65 us; rank 2: 56 / 64, 47 / 67 us; 4,096 rows, rank 32: 69 / 114, 50 / 83 us; 65,536 rows, rank 32:
 // 151 / 883, 82 / 166 us; 589,824 rows, rank 48, FP32: 596 / 1,783 us.
 constexpr long kUdMinRows = 1024;
 // Where the caller asked for 3xTF32 (k_update_tc, FP32 storage): 4,096 rows, rank 32: 50 / 94 us; 131,072 rows:
-// 118 / 218 us.
+// 118 / 218 us.  Below, the split-TF32 kernel that the precision names keeps the first update (1,024 rows, rank 32:
+// 60 / 92 us), for the arithmetic asked for, not for speed.
 constexpr long kUdMinRowsTc = 4096;
 constexpr int kUdDead = 1 << 20;                 // column scale that makes every digit zero
 constexpr int kUdMinExp = -8000;                 // row scale of a zero row

@@ -6,8 +6,9 @@
 //   v = sum_j d_j 256^(NS-1-j),   -128 <= d_j <= 127,
 // NS = 4 digits (30 bits and sign) for FP32 passes and NS = 8 (62 bits and sign) for FP64 passes.
 // Digits are exact in FP16, products of two digits are integers up to 2^14, and the FP32
-// accumulators of tcgen05.mma.kind::f16 sum 256 rows of them without any rounding (every partial sum is
-// an integer of at most 2^22).  The digit products of a chunk are then folded into 64-bit integers.
+// accumulators of tcgen05.mma.kind::f16 sum 1,024 rows of them without any rounding (every partial sum is
+// an integer of at most 2^24: the limit, a longer chunk would round).  The digit products of a chunk are then
+// folded into 64-bit integers.
 // So sum_k v_a v_b comes out exactly, for columns whose entries carry a fixed-point rounding of at most
 // 2^-(8 NS - 1) of their column's largest entry (FP32 2^-31, FP64 2^-63; the storage's own rounding of
 // entries near that size is 2^-25 and 2^-54).  The columns of the transport sum are integer
@@ -15,8 +16,9 @@
 // integer combination of the products of the neighbour blocks, formed without rounding or
 // cancellation (k_xg_combine); the operators' coefficients scale the factor's columns at the end.
 //
-// The factor R with R^T R = G is a Cholesky factor in 128-bit fixed point (xchol.cuh): G is exact and
-// columns are resolved down to about 2^-57 of their norm, as a Householder QR in FP64 resolves them.
+// The factor R with R^T R = G is a Cholesky factor in fixed point (xchol.cuh), 128 bits for FP64 passes and 64 for
+// FP32 ones: G is exact and columns are resolved down to about 2^-57 (2^-27) of their norm, as a Householder QR in
+// FP64 (FP32) resolves them.
 //
 // Why: a Householder TSQR is a chain of reflectors behind block barriers on the FMA pipes; measured
 // at 1,048,576 rows x 160 columns it took 5.3 ms (FP32 leaf) + 2.1 ms (merges) and 91.9 + 17 ms in
@@ -893,7 +895,7 @@ __device__ __forceinline__ void add_shifted(Int192& a, __int128 v, int sh) {  //
 // the right column: gint[word plane][row a][column b], row-major with ldg.  Upper triangle of blocks: the
 // mirrored entry is written too; split: columns of array 1 start at ldg's column 0.
 // unit, coef (nullable): the columns' units and coefficients where the raw columns are the columns.  add: to what
-// is there (rows in several passes; split only).
+// is there (rows in several passes).
 template <int NS>
 __global__ void __launch_bounds__(256) k_xg_sum(const __grid_constant__ XgPlan pl, int ngroups, int split, int ldg,
                                                 size_t plane, const long long* __restrict__ part,
