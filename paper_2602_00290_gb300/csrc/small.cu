@@ -165,15 +165,18 @@ __global__ void k_decide(const double* __restrict__ sigma, int n, int first, int
 // singular value, so every column is cleaned of its components along the larger ones; a column
 // with nothing left (relative remainder <= 1e-12) is replaced by the first canonical vector on a
 // live row (row % rowmod < rowlive) that is independent of the earlier columns.
+// skip (nullable): nothing to do where it is set.
 __global__ void __launch_bounds__(1024) k_orthonormalise(int nv, int ldv, double* __restrict__ V, const int* kptr,
-                                                         int rowmod, const int* rowlive_ptr) {
+                                                         int rowmod, const int* rowlive_ptr,
+                                                         const int* __restrict__ skip) {
+  if (skip && *skip != 0) return;
   __shared__ double red[33];
   __shared__ double h[1024];
   const int k = *kptr;
   const int rowlive = rowlive_ptr ? *rowlive_ptr : rowmod;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nwarps = blockDim.x >> 5;
+  int cand = -1;  // a canonical vector that one column did not take lies in the span of the earlier ones: not tried again
   for (int j = 0; j < k; ++j) {
-    int cand = -1;
     for (int attempt = 0; attempt <= nv; ++attempt) {
       if (attempt > 0) {
         do {
@@ -186,6 +189,7 @@ __global__ void __launch_bounds__(1024) k_orthonormalise(int nv, int ldv, double
       double n0 = 0.0;
       for (int i = threadIdx.x; i < nv; i += blockDim.x) n0 += V[(size_t)i * ldv + j] * V[(size_t)i * ldv + j];
       n0 = sqrt(block_sum(n0, red));
+      if (n0 == 0.0) continue;
       for (int pass = 0; pass < 2; ++pass) {
         for (int i2 = warp; i2 < j; i2 += nwarps) {
           double sacc = 0.0;
@@ -221,8 +225,8 @@ __global__ void __launch_bounds__(1024) k_orthonormalise(int nv, int ldv, double
 // one lane per row, warp shuffles for norms; no block-wide barriers.  Same algorithm and outputs.
 __device__ void cgs2_warp_staged(int nv, int k, int rowmod, int rowlive, double* V, double* h) {
   const int lane = threadIdx.x & 31;
+  int cand = -1;  // a canonical vector that one column did not take lies in the span of the earlier ones: not tried again
   for (int j = 0; j < k; ++j) {
-    int cand = -1;
     for (int attempt = 0; attempt <= nv; ++attempt) {
       if (attempt > 0) {
         do {
@@ -234,6 +238,7 @@ __device__ void cgs2_warp_staged(int nv, int k, int rowmod, int rowlive, double*
       }
       double x = (lane < nv) ? V[lane * 33 + j] : 0.0;
       const double n0 = sqrt(warp_sum(x * x));
+      if (n0 == 0.0) continue;
       for (int pass = 0; pass < 2; ++pass) {
         // both dependent FP64 chains in four partial sums
         double h0 = 0.0, h1 = 0.0, h2 = 0.0, h3 = 0.0;
@@ -330,10 +335,9 @@ __global__ void __launch_bounds__(128) k_orthonormalise_polar(int nv, int ldv, d
   if (tid == 0) {
     double m = 0.0;
     for (int w = 0; w < (int)(blockDim.x >> 5); ++w) m = (emax[w] > m || emax[w] != emax[w]) ? emax[w] : m;
-    // no step below the FP64 round-off of a k-term sum; one from e <= 1e-8; two from e <= 1e-4;
-    // otherwise Gram-Schmidt (-1)
-    const double floor64 = 8.0 * 2.220446049250313e-16 * (k > 1 ? k : 1);
-    nsteps = (m <= floor64) ? 0 : (m <= 1e-8) ? 1 : (m <= 1e-4) ? 2 : -1;
+    // one step from e <= 1e-8 (also near round-off: a Jacobi sweep stops at cosines of 2 n eps, and left without
+    // a step 32 columns were 11 times as far from orthonormal); two from e <= 1e-4; otherwise Gram-Schmidt (-1)
+    nsteps = (m <= 1e-8) ? 1 : (m <= 1e-4) ? 2 : -1;
   }
   __syncthreads();
   const int ns = nsteps;
@@ -381,6 +385,25 @@ __global__ void __launch_bounds__(128) k_orthonormalise_polar(int nv, int ldv, d
     const int i = idx / ldv, c = idx - (idx / ldv) * ldv;
     Vg[idx] = V[i * 33 + c];
   }
+}
+
+// One such step for more than 32 columns as a product: M <- (3 I - G) / 2 over the first k columns for G = V^T V
+// (n x n, overwritten), *done = 1; where an entry of G - I is beyond 1e-8, M <- I and *done = 0 (Gram-Schmidt).
+__global__ void __launch_bounds__(1024) k_polar_matrix(int n, double* __restrict__ G, const int* kptr,
+                                                       int* __restrict__ done) {
+  const int k = *kptr;
+  bool far = false;
+  for (int idx = threadIdx.x; idx < n * n; idx += blockDim.x) {
+    const int a = idx / n, b = idx - (idx / n) * n;
+    if (a < k && b < k) far = far || !(fabs(G[idx] - (a == b ? 1.0 : 0.0)) <= 1e-8);
+  }
+  far = __syncthreads_or(far) != 0;
+  for (int idx = threadIdx.x; idx < n * n; idx += blockDim.x) {
+    const int a = idx / n, b = idx - (idx / n) * n;
+    const bool in = a < k && b < k && !far;
+    G[idx] = a == b ? (in ? 1.5 - 0.5 * G[idx] : 1.0) : in ? -0.5 * G[idx] : 0.0;
+  }
+  if (threadIdx.x == 0) *done = far ? 0 : 1;
 }
 
 // Mixed-path form of k_orthonormalise_polar, for columns that are FP32-accurate right singular
@@ -2121,7 +2144,7 @@ static tt_status small_round_mixed3(cudaStream_t s, int num_sms, const SmallJob&
     else if (n2 <= 32)
       k_orthonormalise_polar_mixed<<<1, 128, 0, s>>>(n2, n2, V2, &j.ctrl->k[1], n2, nullptr);
     else
-      k_orthonormalise<<<1, 1024, 0, s>>>(n2, n2, V2, &j.ctrl->k[1], n2, nullptr);
+      k_orthonormalise<<<1, 1024, 0, s>>>(n2, n2, V2, &j.ctrl->k[1], n2, nullptr, nullptr);
     count_launch();
     small_gemm_pair<double, double>(s, R * n1, K2, n2, Y, j.B0, n2, 1, V2, n2, 1, Y2, B0p, K2, &j.ctrl->k[1]);
   }
@@ -2193,9 +2216,18 @@ tt_status small_round(cudaStream_t s, int num_sms, const SmallJob& j, Bump& ws) 
     // the only bond: SVD of Y (R x n1)
     double* sig = ws.take<double>(n1);
     double* V = nullptr;
+    bool normalised = false;  // columns of V from the cluster Jacobi
+    double *G = nullptr, *Vp = nullptr;
+    int* done = nullptr;
     if (!j.no_xg && n1 <= kJcMaxN && xg_fits<double>(SrcRows<double>{Y, n1}, LivePattern{nullptr, n1, 1, 0}, R)) {
       int* perm = ws.take<int>(n1);
       double* tmp = ws.take<double>((size_t)n1 * n1);
+      normalised = true;
+      if (n1 > 32) {
+        G = ws.take<double>((size_t)n1 * n1);
+        Vp = ws.take<double>((size_t)n1 * n1);
+        done = ws.take<int>(1);
+      }
       st = svd_right_xg<true>(s, num_sms, SrcRows<double>{Y, n1}, R, n1, ws, &V, nullptr, sig, perm, j.ctrl);
       if (st != TT_OK || ws.dry) return st;
       k_sort_cols<<<1, 1024, 0, s>>>(n1, n1, n1, sig, V, tmp); count_launch();
@@ -2206,6 +2238,19 @@ tt_status small_round(cudaStream_t s, int num_sms, const SmallJob& j, Bump& ws) 
     }
     k_decide<<<1, 32, 0, s>>>(sig, n1, 1, 2, j.tol, j.rmax, j.K1cap, j.nrowsZ, j.lp.r_ptr, j.lp.nblk,
                               j.lp.nextra, 1, nullptr, 0, 0, nullptr, 0, n1, j.ctrl, 0, nullptr); count_launch();
+    // The cluster Jacobi's normalised columns are orthogonal to its stopping cosine (2 n eps), those below the
+    // round-off of the largest not even to that, and zero where the factor is: the angular core is right-orthonormal
+    // after a polar step, or Gram-Schmidt.  (The accumulated rotations of svd_right are, to round-off.)  A step of
+    // the 1-D slab, FP64: 582 / 920 / 2,312 us without it and 614 / 950 / 2,352 us with it at 8 / 16 / 40 ordinates.
+    if (normalised && n1 <= 32) {
+      k_orthonormalise_polar<<<1, 128, 0, s>>>(n1, n1, V, &j.ctrl->k[0], n1, nullptr); count_launch();
+    } else if (normalised) {
+      small_gemm<double, double>(s, n1, n1, n1, V, 1, n1, V, n1, 1, G, n1, nullptr, nullptr);
+      k_polar_matrix<<<1, 1024, 0, s>>>(n1, G, &j.ctrl->k[0], done); count_launch();
+      small_gemm<double, double>(s, n1, n1, n1, V, n1, 1, G, n1, 1, Vp, n1, nullptr, nullptr);
+      k_orthonormalise<<<1, 1024, 0, s>>>(n1, n1, Vp, &j.ctrl->k[0], n1, nullptr, done); count_launch();
+      V = Vp;
+    }
     small_gemm<double, double>(s, R, j.K1cap, n1, j.B0, n1, 1, V, n1, 1, j.W, j.K1cap, &j.ctrl->k[0], nullptr);
     k_write_cores2<<<(j.K1cap * n1 + 255) / 256, 256, 0, s>>>(n1, j.K1cap, V, j.ctrl, j.core1); count_launch();
     cudaMemcpyAsync(j.Bnew, j.core1, sizeof(double) * (size_t)j.K1cap * n1, cudaMemcpyDeviceToDevice, s);
