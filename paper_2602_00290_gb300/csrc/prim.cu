@@ -70,7 +70,8 @@ __global__ void __launch_bounds__(256) k_transport_Z(long N, SrcStencil<S> src, 
     if (mine && c < R && r > 0) cc = src.col(c);
     // coefficient of the (second) difference
     const double lam = cc.kind == 4 ? -0.5 * cc.lam : cc.kind == 5 ? 0.5 * cc.lam : -cc.lam;
-    const float lh = (float)lam, ll = (float)(lam - (double)lh);
+    // (a coefficient whose parts would be subnormal: zero, which sends every entry to FP64)
+    const float lh = fabs(lam) > 1e-25 ? (float)lam : 0.0f, ll = (float)(lam - (double)lh);
     const bool lo = cc.kind >= 4 || (cc.kind == 1 && cc.w > 0), hi = cc.kind >= 4 || (cc.kind == 1 && cc.w <= 0);
     for (long row0 = (long)blockIdx.x * kTrRows; row0 < N; row0 += (long)gridDim.x * kTrRows) {
       __syncthreads();
