@@ -287,21 +287,25 @@ __device__ void cgs2_warp_staged(int nv, int k, int rowmod, int rowlive, double*
 // 1e-8 (FP64 Jacobi) and two for FP32-accurate columns.  The span of the columns is unchanged and
 // the columns move by O(e).  Other inputs (a vanishing or far from orthogonal column) take the
 // column-by-column Gram-Schmidt of cgs2_warp_staged, which also replaces dependent columns.
-// Four warps compute V^T V and the update as small matrix products in shared memory: no
+// Eight warps compute V^T V and the update as small matrix products in shared memory: no
 // dependent chain longer than nv, against the column-by-column chains of Gram-Schmidt.
-__global__ void __launch_bounds__(128) k_orthonormalise_polar(int nv, int ldv, double* __restrict__ Vg,
+__global__ void __launch_bounds__(256) k_orthonormalise_polar(int nv, int ldv, double* __restrict__ Vg,
                                                               const int* kptr, int rowmod, const int* rowlive_ptr) {
   __shared__ double V[32 * 33];
   __shared__ double G[32 * 33];
   __shared__ double h[32];
-  __shared__ double emax[4];
+  __shared__ float Vf[32 * 33];
+  __shared__ float Ef[32 * 33];
+  __shared__ double emax[8];
   __shared__ int nsteps;
+  __shared__ bool fine;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int k = *kptr;
   const int rowlive = rowlive_ptr ? *rowlive_ptr : rowmod;
   for (int idx = tid; idx < nv * ldv; idx += blockDim.x) {
     const int i = idx / ldv, c = idx - (idx / ldv) * ldv;
     V[i * 33 + c] = Vg[idx];
+    Vf[i * 33 + c] = (float)Vg[idx];
   }
   __syncthreads();
   // G = V^T V over the first k columns; returns max |G - I| over this thread's entries
@@ -320,6 +324,7 @@ __global__ void __launch_bounds__(128) k_orthonormalise_polar(int nv, int ldv, d
       for (; i < nv; ++i) g0 += V[i * 33 + a] * V[i * 33 + b];
       const double g = (g0 + g1) + (g2 + g3);
       G[a * 33 + b] = g;
+      Ef[a * 33 + b] = (float)(g - (a == b ? 1.0 : 0.0));
       const double d = fabs(g - (a == b ? 1.0 : 0.0));
       e = (d > e || d != d) ? d : e;  // a NaN counts as far from orthonormal
     }
@@ -338,6 +343,7 @@ __global__ void __launch_bounds__(128) k_orthonormalise_polar(int nv, int ldv, d
     // one step from e <= 1e-8 (also near round-off: a Jacobi sweep stops at cosines of 2 n eps, and left without
     // a step 32 columns were 11 times as far from orthonormal); two from e <= 1e-4; otherwise Gram-Schmidt (-1)
     nsteps = (m <= 1e-8) ? 1 : (m <= 1e-4) ? 2 : -1;
+    fine = m <= 1e-10;
   }
   __syncthreads();
   const int ns = nsteps;
@@ -345,15 +351,31 @@ __global__ void __launch_bounds__(128) k_orthonormalise_polar(int nv, int ldv, d
     if (warp == 0) cgs2_warp_staged(nv, k, rowmod, rowlive, V, h);
     __syncthreads();
   }
-  for (int step = 0; step < ns; ++step) {
+  if (ns == 1 && fine) {
+    // V - V E / 2 for E = G - I of at most 1e-10: the product in FP32, 2^-24 of it is below 2^-56 of V (in FP64, with
+    // four warps, the kernel took 51 us at 32 columns)
+    for (int idx = tid; idx < nv * k; idx += blockDim.x) {
+      const int i = idx / k, b = idx - (idx / k) * k;
+      float s0 = 0.f, s1 = 0.f;
+      int a = 0;
+      for (; a + 1 < k; a += 2) {
+        s0 = fmaf(Vf[i * 33 + a], Ef[a * 33 + b], s0);
+        s1 = fmaf(Vf[i * 33 + a + 1], Ef[(a + 1) * 33 + b], s1);
+      }
+      if (a < k) s0 = fmaf(Vf[i * 33 + a], Ef[a * 33 + b], s0);
+      V[i * 33 + b] -= 0.5 * (double)(s0 + s1);
+    }
+    __syncthreads();
+  }
+  for (int step = 0; step < (fine ? 0 : ns); ++step) {
     if (step > 0) {
       (void)gram();
       __syncthreads();
     }
-    // V[i][b] <- 1.5 V[i][b] - 0.5 sum_a V[i][a] G[a][b] (b < k): nv k <= 1024 entries, 8 a thread
-    double w[8];
+    // V[i][b] <- 1.5 V[i][b] - 0.5 sum_a V[i][a] G[a][b] (b < k): nv k <= 1024 entries, 4 a thread
+    double w[4];
 #pragma unroll
-    for (int r = 0; r < 8; ++r) {
+    for (int r = 0; r < 4; ++r) {
       const int idx = tid + r * (int)blockDim.x;
       w[r] = 0.0;
       if (idx < nv * k) {
@@ -372,7 +394,7 @@ __global__ void __launch_bounds__(128) k_orthonormalise_polar(int nv, int ldv, d
     }
     __syncthreads();
 #pragma unroll
-    for (int r = 0; r < 8; ++r) {
+    for (int r = 0; r < 4; ++r) {
       const int idx = tid + r * (int)blockDim.x;
       if (idx < nv * k) {
         const int i = idx / k, b = idx - (idx / k) * k;
@@ -2140,7 +2162,7 @@ static tt_status small_round_mixed3(cudaStream_t s, int num_sms, const SmallJob&
     // one polar step; the mixed path's FP32-accurate small columns are only ~1e-2 orthogonal
     // (the FP32 sweep stops at its round-off floor): their polar steps start in FP32
     if (n2 <= 32 && F64)
-      k_orthonormalise_polar<<<1, 128, 0, s>>>(n2, n2, V2, &j.ctrl->k[1], n2, nullptr);
+      k_orthonormalise_polar<<<1, 256, 0, s>>>(n2, n2, V2, &j.ctrl->k[1], n2, nullptr);
     else if (n2 <= 32)
       k_orthonormalise_polar_mixed<<<1, 128, 0, s>>>(n2, n2, V2, &j.ctrl->k[1], n2, nullptr);
     else
@@ -2241,9 +2263,9 @@ tt_status small_round(cudaStream_t s, int num_sms, const SmallJob& j, Bump& ws) 
     // The cluster Jacobi's normalised columns are orthogonal to its stopping cosine (2 n eps), those below the
     // round-off of the largest not even to that, and zero where the factor is: the angular core is right-orthonormal
     // after a polar step, or Gram-Schmidt.  (The accumulated rotations of svd_right are, to round-off.)  A step of
-    // the 1-D slab, FP64: 582 / 920 / 2,312 us without it and 614 / 950 / 2,352 us with it at 8 / 16 / 40 ordinates.
+    // the 1-D slab, FP64: 582 / 920 / 2,312 us without it and 607 / 942 / 2,355 us with it at 8 / 16 / 40 ordinates.
     if (normalised && n1 <= 32) {
-      k_orthonormalise_polar<<<1, 128, 0, s>>>(n1, n1, V, &j.ctrl->k[0], n1, nullptr); count_launch();
+      k_orthonormalise_polar<<<1, 256, 0, s>>>(n1, n1, V, &j.ctrl->k[0], n1, nullptr); count_launch();
     } else if (normalised) {
       small_gemm<double, double>(s, n1, n1, n1, V, 1, n1, V, n1, 1, G, n1, nullptr, nullptr);
       k_polar_matrix<<<1, 1024, 0, s>>>(n1, G, &j.ctrl->k[0], done); count_launch();
