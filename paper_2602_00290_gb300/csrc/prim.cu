@@ -31,7 +31,13 @@ __device__ __forceinline__ double tr_scaled(double lam, float, float, double a, 
 // (t = 0 state, t = 1..nterm operator images) and the nbc inflow columns after them.  A thread keeps
 // one column (its operator is looked up once), a CTA takes 64 rows at a time (their neighbour flags are
 // formed once, by 64 threads), four rows of a thread in flight.  1,048,576 x 81 FP32: 0.37 ms (340 MB written); with a
-// thread per entry, which divided for its row, column and neighbours in 64 bits and scaled in FP64: 1.47 ms.
+// thread per entry, which divides for its row, column and neighbours in 64 bits and scales in FP64: 1.47 ms.
+// Below 32,768 rows (FP64: 64 a CTA) a CTA takes fewer rows, so that all of them have some: 7,488 x 180 FP32 37 -> 29 us,
+// 16,384 x 180 FP64 62 -> 48.  A thread per entry (k_transport_entry) stays where it is faster, thread per entry / columns:
+//   FP32, up to 5 x 2^16 entries: 576 x 100 19 / 25 us, 2,048 x 100 20 / 26, 7,488 x 40 20 / 22, 7,488 x 72 26 / 22
+//   FP64 central differences, up to 2^20: 576 x 180 24 / 46, 7,488 x 72 21 / 29, 16,384 x 72 32 / 30, 55,296 x 27 39 / 35
+//   FP64 upwind, up to 6 x 2^20 or where the columns leave a fifth of a CTA idle: 55,296 x 15 25 / 27, 131,072 x 40 78 /
+//     83, 442,368 x 15 102 / 100, 442,368 x 40 258 / 240; 100 columns: 131,072 173 / 193, 1,048,576 1,316 / 1,373
 constexpr int kTrRows = 64;
 // SrcStencil::row_flags in 32 bits where the rows allow it (64-bit division runs on the FP64 pipe).
 template <typename S>
@@ -47,10 +53,51 @@ __device__ __forceinline__ unsigned tr_flags(const SrcStencil<S>& src, long k, l
   return f | (((unsigned)k % (unsigned)src.G) << 8);
 }
 template <typename S>
+__global__ void __launch_bounds__(256) k_transport_entry(long N, SrcStencil<S> src, const int* __restrict__ rank_in,
+                                                         S* __restrict__ Zo, int ldo, int nbc,
+                                                         const int* __restrict__ rank_in2, int rcapo2, int,
+                                                         int* status) {
+  const int r = rank_in[1];
+  const int R = (src.nterm + 1) * r + nbc;
+  bool over = R > ldo;
+  if (rank_in2) over = over || ((src.nterm + 1) * (*rank_in2) + nbc > rcapo2);
+  if (over) {
+    if (blockIdx.x == 0 && threadIdx.x == 0) latch(status, TT_ERR_CAPACITY);
+    return;
+  }
+  src.rcap = r > 0 ? r : 1;
+  const long tot = N * (long)ldo;
+  for (long idx = blockIdx.x * (long)blockDim.x + threadIdx.x; idx < tot; idx += (long)gridDim.x * blockDim.x) {
+    const long k = idx / ldo;
+    const int c = (int)(idx - k * ldo);
+    S v = S(0);
+    if (c < R && r > 0) {
+      const auto cc = src.col(c);
+      if (sizeof(S) == 8 || (cc.kind != 1 && cc.kind < 4)) {
+        v = (S)src.load(cc, k);
+      } else {  // as k_transport_Z forms it
+        const double lam = cc.kind == 4 ? -0.5 * cc.lam : cc.kind == 5 ? 0.5 * cc.lam : -cc.lam;
+        const float lh = fabs(lam) > 1e-25 ? (float)lam : 0.0f, ll = (float)(lam - (double)lh);
+        const unsigned f = tr_flags(src, k, N) >> (2 * cc.ax);
+        const S* z = src.Z + k * src.ldz + cc.q;
+        const long st = cc.s * src.ldz;
+        const bool both = cc.kind >= 4;
+        const S zl = (both || cc.w > 0) && (f & 1u) ? z[-st] : S(0), zh = (both || cc.w <= 0) && (f & 2u) ? z[st] : S(0);
+        const S x = !both && cc.w > 0 ? z[0] : zh;
+        const S y = cc.kind == 5 ? S(-2) * z[0] : !both && cc.w <= 0 ? -z[0] : -zl;
+        v = tr_scaled(lam, lh, ll, x, y, cc.kind == 5 ? zl : S(0));
+      }
+    }
+    Zo[idx] = v;
+  }
+}
+template <typename S, int ROWS>
 __global__ void __launch_bounds__(256) k_transport_Z(long N, SrcStencil<S> src, const int* __restrict__ rank_in,
                                                      S* __restrict__ Zo, int ldo, int nbc,
-                                                     const int* __restrict__ rank_in2, int rcapo2, int* status) {
+                                                     const int* __restrict__ rank_in2, int rcapo2, int nrow,
+                                                     int* status) {
   __shared__ unsigned fl[kTrRows];
+  const int rows = ROWS ? ROWS : nrow;
   const int r = rank_in[1];
   const int R = (src.nterm + 1) * r + nbc;
   bool over = R > ldo;
@@ -73,12 +120,12 @@ __global__ void __launch_bounds__(256) k_transport_Z(long N, SrcStencil<S> src, 
     // (a coefficient whose parts would be subnormal: zero, which sends every entry to FP64)
     const float lh = fabs(lam) > 1e-25 ? (float)lam : 0.0f, ll = (float)(lam - (double)lh);
     const bool lo = cc.kind >= 4 || (cc.kind == 1 && cc.w > 0), hi = cc.kind >= 4 || (cc.kind == 1 && cc.w <= 0);
-    for (long row0 = (long)blockIdx.x * kTrRows; row0 < N; row0 += (long)gridDim.x * kTrRows) {
+    for (long row0 = (long)blockIdx.x * rows; row0 < N; row0 += (long)gridDim.x * rows) {
       __syncthreads();
-      for (int m = tid; m < kTrRows; m += 256) fl[m] = row0 + m < N ? tr_flags(src, row0 + m, N) : 0u;
+      for (int m = tid; m < rows; m += 256) fl[m] = row0 + m < N ? tr_flags(src, row0 + m, N) : 0u;
       __syncthreads();
       if (!mine) continue;
-      const int nr = (int)(N - row0 < kTrRows ? N - row0 : kTrRows);
+      const int nr = (int)(N - row0 < rows ? N - row0 : rows);
       const S* z = src.Z + row0 * src.ldz + cc.q;
       S* o = Zo + row0 * ldo + c;
       const long st = cc.s * src.ldz;
@@ -315,8 +362,20 @@ tt_status apply_transport_impl(tt_context* ctx, const tt_plan* p, const tt_tenso
   src.nax = p->ndim;
   const long N = in->n[0];
   const int rcapo2 = (d == 3) ? out->rcap[2] : 1;
-  k_transport_Z<S><<<8 * (unsigned)ctx->num_sms, 256, 0, s>>>(N, src, in->rank, (S*)out->core[0], out->rcap[1], p->nbc,
-                                        d == 3 ? in->rank + 2 : nullptr, rcapo2, &ctx->ctrl->status); count_launch();
+  // Which kernel: see k_transport_Z
+  const long grid = 8L * ctx->num_sms, tot = N * (long)out->rcap[1];
+  const int cols = out->rcap[1] < 256 ? out->rcap[1] : 256;
+  bool wide = false;  // central differences
+  for (int t = 0; t < p->nterm; ++t) wide = wide || p->term_w[t] > 1 || p->term_w[t] < -1;
+  const bool entry = sizeof(S) == 4 ? tot <= 5 * (1L << 16)
+                     : wide         ? tot <= (1L << 20)
+                                    : tot <= 6 * (1L << 20) || 256 / cols * cols < 208;
+  const bool full = N >= (sizeof(S) == 4 ? 32768L : grid * kTrRows);
+  const int rows = full ? kTrRows : N <= 4 * grid ? 4 : (int)((N + grid - 1) / grid);
+  auto kern = entry ? k_transport_entry<S> : full ? k_transport_Z<S, kTrRows> : k_transport_Z<S, 0>;
+  kern<<<(unsigned)(entry ? 1024 : grid), 256, 0, s>>>(N, src, in->rank, (S*)out->core[0], out->rcap[1], p->nbc,
+                                                       d == 3 ? in->rank + 2 : nullptr, rcapo2, rows, &ctx->ctrl->status);
+  count_launch();
   k_transport_small<S><<<64, 256, 0, s>>>(d, p->nterm, p->nbc, p->n1, p->n2, (const S*)in->core[1],
                                           d == 3 ? (const S*)in->core[2] : nullptr, in->rcap[1],
                                           d == 3 ? in->rcap[2] : 1, in->rank, (S*)out->core[1],
